@@ -78,7 +78,7 @@ struct PipePlan {
   int use = 0, T = 1, m = 1, maxm = 8;
   int cw = 32, W = 1;  // columns per tile (32, or 16 for long lines); consumer warps
   int box_rows = 0, nbox = 0, rows_per_tile = 0, pitch = 0;
-  int stages = 0, grid = 0;
+  int stages = 0, ctas = 1, grid = 0;  // ctas: per SM
   int64_t stage_elems = 0, ntiles = 0;
   size_t smem = 0;
   CUtensorMap map[2]{};  // y/z: [0] the field, [1] the adjoint field
@@ -125,11 +125,9 @@ struct biofvm {
   // FP32 fields whose rows (nx*S elements) are not 16-byte multiples, which the TMA copies
   // need: biofvm_step runs the pipelined sweeps on a row-padded working copy (rows gpitch
   // elements apart, the padding zero), copied in at the start of the call and back at its
-  // end.  ppx: the plans over that copy; tabP / tabTP: their axis tables when a plan's chunk
-  // partition differs from the one the handle's own tables follow (tabP_own)
+  // end.  ppx: the plans over that copy; tabP / tabTP: the axis tables of their partitions
   int pitched = 0, gpitch = 0, pitched_enabled = 1;
   DevBuf prow, tabP[3], tabTP[3];
-  int tabP_own[3] = {0, 0, 0};
   PipePlan ppx[3];
   StreamPlan sp[3];
   int num_sms = 0;
@@ -424,33 +422,34 @@ bool encode_pipe_map(biofvm *h, PipePlan &p, int axis, int buf, void *field, int
   return p.have_map[buf] != 0;
 }
 
-// Bank-conflict degree of 32 lanes reading column c at (c/S)*pitch + c%S
-// (x tiles, pitch in elements): the largest number of distinct 4-byte words a
-// bank serves (lanes on one word share it: 16-bit elements pair up), or for
-// FP64 the largest number of lanes sharing a bank pair within a half warp.
-// half_off >= 0 (tiles of 16 columns): lanes 16..31 read columns 0..15 of the
-// next chunk, half_off elements further on.
-int x_tile_conflicts(int64_t pitch, int S, int lanes, size_t esz, int64_t half_off = -1) {
-  int worst = 0;
-  if (esz == 8) {
-    for (int half = 0; half < 2; half++) {
-      int cnt[16] = {0};
-      for (int c = half * 16; c < std::min(lanes, half * 16 + 16); c++)
-        worst = std::max(worst, ++cnt[(int)(((c / S) * pitch + c % S) & 15)]);
+// Shared-memory wavefronts of one warp access of the pipelined x tile at row
+// pitch `pitch` (elements): lane l reads column pair l % (cw/2) of its chunk, m
+// positions from the next lane group's, as pipe.cuh does -- S = 1: four
+// consecutive positions of a row, S = 2: two positions of both substrates, even
+// S: a pair of substrates, else one column.  The hardware serves 128 bytes of
+// lanes at a time; a group of lanes costs the most distinct words in one bank.
+int x_tile_wavefronts(int64_t pitch, int S, int cw, int m, size_t esz) {
+  const bool wide = S == 1 || S == 2;
+  const bool even = S == 2 || S == 4 || S == 8;
+  const int width = (int)esz * (wide ? 4 : even ? 2 : 1);  // bytes a lane reads
+  const int pw = cw / 2, per = std::max(1, std::min(32, 128 / width)), ncol = cw / S * S;
+  int total = 0;
+  for (int g = 0; g < 32; g += per) {
+    std::vector<int64_t> words[32];
+    size_t worst = 0;
+    for (int l = g; l < std::min(32, g + per); l++) {
+      int c = S == 1 ? l % pw : 2 * (l % pw);
+      if (c >= ncol) c = 0;
+      const int64_t byte = ((c / S) * pitch + c % S + (int64_t)(l / pw) * m * S) * (int64_t)esz;
+      for (int64_t w = byte / 4; w <= (byte + width - 1) / 4; w++) {
+        std::vector<int64_t> &v = words[w & 31];
+        if (std::find(v.begin(), v.end(), w) == v.end()) v.push_back(w);
+        worst = std::max(worst, v.size());
+      }
     }
-    return worst;
+    total += (int)worst;
   }
-  std::vector<int64_t> words[32];
-  for (int l = 0; l < 32; l++) {
-    const int c = half_off >= 0 ? (l & 15) : l;
-    if (c >= lanes) continue;
-    const int64_t e = (c / S) * pitch + c % S + (half_off >= 0 && l >= 16 ? half_off : 0);
-    const int64_t word = e * (int64_t)esz / 4;
-    std::vector<int64_t> &w = words[word & 31];
-    if (std::find(w.begin(), w.end(), word) == w.end()) w.push_back(word);
-    worst = std::max(worst, (int)w.size());
-  }
-  return worst;
+  return total;
 }
 
 // Plan the pipelined sweep of axis 0 (x), 1 (y) or 2 (z) over `field`, whose
@@ -461,63 +460,28 @@ int x_tile_conflicts(int64_t pitch, int S, int lanes, size_t esz, int64_t half_o
 void plan_pipe(biofvm *h, int axis, PipePlan &p, int64_t gp, void *field) {
   p = PipePlan{};
   const int64_t nx = h->g.nx, ny = h->g.ny, nz = h->g.nz, S = h->g.n_sub;
-  const size_t esz = h->esz, csz = h->csz;
+  const size_t esz = h->esz;
   const int n = axis_len(h, axis);
   if (h->prec == BIOFVM_FP64) return;  // FP64 streams whole lines instead
-  const bool h16 = esz == 2;  // 16-bit storage: chunk capacities 32 and 64 compiled
   for (int cw : {32, 16}) {
     if (h->pipe_cw && cw != h->pipe_cw) continue;
     PipePlan q{};
     q.cw = cw;
-    const int cpw = 32 / cw;
+    const int cpw = 64 / cw;  // chunks per consumer warp
     const int extra = axis == 0 ? 2 : 1;  // warps besides the consumers: producer (+ preparer)
-    ColPlan cp;
-    if (h->pipe_chunk > 0) {  // chunk length chosen by the caller (tuning)
-      if (!plan_col(n, false, cp, std::min(h->pipe_chunk, n))) continue;
-    } else if (cw == 32) {
-      // a field that stays in L2 makes the sweep latency-bound: there the shortest chunk, 16
-      // then 24 positions, whose CTA fits (more consumer warps per SM; measured: 250^3 x 1
-      // z-sweep 0.036 against 0.050 ms); in the HBM-bound regime chunks of 32 (at 256^3 x 4
-      // chunks of 16 took the x-sweep from 0.139 to 0.211 ms)
-      const bool l2_resident = (double)h->nel * (double)esz <= 96.0e6;
-      bool shortc = false;
-      for (int target : {16, 24}) {
-        const int T = (n + target - 1) / target;
-        if (!l2_resident || h16 || T < 2 || (T + extra) * 32 > pipe_max_threads_f32(target))
-          continue;
-        cp.T = T;
-        cp.m = target;
-        cp.maxm = target;
-        shortc = true;
-        break;
-      }
-      if (!shortc && !plan_col(n, false, cp)) continue;
-    } else {  // 16 columns: chunks of 32 or 64 (the capacities compiled for them)
-      bool found = false;
-      for (int target : {32, 64}) {
-        const int T = std::max(1, (n + target - 1) / target);
-        const int m = T == 1 ? n : target;
-        const int maxm = pick_maxm(m, false);
-        if (maxm != 32 && maxm != 64) continue;
-        if (((T + 1) / 2 + extra) * 32 > pipe_max_threads_f32(maxm)) continue;
-        cp.T = T;
-        cp.m = m;
-        cp.maxm = maxm;
-        found = true;
-        break;
-      }
-      if (!found) continue;
+    // chunks of exactly the capacity (the last one shorter), 16 positions where their warps fit
+    // in a CTA, else 24 (positions past the line's end have zero coefficients)
+    bool found = false;
+    for (int target : {16, 24}) {
+      const int want = h->pipe_chunk > 0 ? h->pipe_chunk : target;
+      q.m = q.maxm = want <= 8 && cw == 32 ? 8 : want <= 16 ? 16 : 24;
+      q.T = (n + q.m - 1) / q.m;
+      q.W = (q.T + cpw - 1) / cpw;
+      if (q.W + extra > pipe_sm_warps(q.maxm)) continue;
+      found = true;
+      break;
     }
-    if (h16 && cp.maxm < 32) cp.maxm = 32;  // short chunks run on the guarded path
-    if (h16 && cp.maxm > 64) continue;
-    if (cw == 16 && cp.maxm != 32 && cp.maxm != 64) continue;
-    // chunks above 64 registers spill (measured with -Xptxas -v): 16-column tiles instead
-    if (cw == 32 && cp.maxm > 64 && h->pipe_chunk <= 0) continue;
-    const int W = (cp.T + cpw - 1) / cpw;  // consumer warps
-    if ((W + extra) * 32 > pipe_max_threads_f32(cp.maxm)) continue;
-    q.T = cp.T;
-    q.m = cp.m;
-    q.maxm = cp.maxm;
+    if (!found) continue;
     if (axis == 0) {
       if ((gp * (int64_t)esz) % 16 != 0 || S > cw) continue;
       q.rows_per_tile = (int)(cw / S);
@@ -526,9 +490,7 @@ void plan_pipe(biofvm *h, int axis, PipePlan &p, int64_t gp, void *field) {
       const int align = (int)(16 / esz);
       int best = 1 << 30;
       for (int64_t pitch = gp; pitch <= gp + 64; pitch += align) {
-        const int d = cw == 16 ? x_tile_conflicts(pitch, (int)S, q.rows_per_tile * (int)S, esz,
-                                                  (int64_t)q.m * S)
-                               : x_tile_conflicts(pitch, (int)S, q.rows_per_tile * (int)S, esz);
+        const int d = x_tile_wavefronts(pitch, (int)S, cw, q.m, esz);
         if (d < best) {
           best = d;
           q.pitch = (int)pitch;
@@ -557,15 +519,22 @@ void plan_pipe(biofvm *h, int axis, PipePlan &p, int64_t gp, void *field) {
       if (q.ntiles > (int64_t)0x7fffffff) return;  // tiles are indexed in 32 bits
     }
     const size_t stage = (size_t)q.stage_elems * esz;
-    const size_t tab = (size_t)pipe_tab_elems_host(n, (int)S) * csz + 16;  // + alignment
-    // carry exchange [2][W*32], carry weights [T][T][S], alignment, mbarriers
-    // (mbarriers: full, done, ready per stage, at most 8 stages)
-    const size_t scratch = (2 * (size_t)W * 32 + (size_t)q.T * q.T * S) * csz + 16 + 3 * 8 * 8;
-    for (int ns = std::max(2, std::min(h->pipe_ns, 8)); ns >= 2 && !q.stages; ns--)  // the constants always staged
-      if (ns * stage + tab + scratch <= kMaxDynamicSmem) q.stages = ns;
+    const size_t tab = (size_t)pipe_tab_pairs(q.maxm, (int)S, q.W, cpw) * 8 + 16;  // + alignment
+    // carry exchange [2][W][cw/2] pairs; mbarriers: full, done, ready per stage, at most 8 stages
+    const size_t scratch = 2 * (size_t)q.W * (cw / 2) * 8 + 3 * 8 * 8;
+    // As many CTAs per SM as the registers take, while each keeps three stages (256 positions:
+    // two CTAs of 9 warps); else one with as many stages as fit.
+    const int most = std::max(2, std::min(h->pipe_ns, 8));
+    for (int c = std::max(1, pipe_sm_warps(q.maxm) / (q.W + extra)); c >= 1 && !q.stages; c--) {
+      const size_t room = std::min(kMaxDynamicSmem, (kMaxDynamicSmem + 1024) / c - 1024);
+      for (int ns = most; ns >= (c > 1 ? std::min(3, most) : 2) && !q.stages; ns--)
+        if (ns * stage + tab + scratch <= room) {
+          q.stages = ns;
+          q.ctas = c;
+        }
+    }
     if (!q.stages) continue;
     q.smem = q.stages * stage + tab + scratch;
-    q.W = W;
     p = q;
     break;
   }
@@ -586,12 +555,7 @@ void plan_pipe(biofvm *h, int axis, PipePlan &p, int64_t gp, void *field) {
     p.use = 0;
     return;
   }
-  const int threads = (p.W + (axis == 0 ? 2 : 1)) * 32;
-  const int regs = p.maxm + 96;
-  int per_sm = (int)std::min<size_t>({kMaxDynamicSmem / p.smem, (size_t)(2048 / threads),
-                                      (size_t)(65536 / (threads * regs))});
-  per_sm = std::max(per_sm, 1);
-  p.grid = (int)std::min<int64_t>(p.ntiles, (int64_t)h->num_sms * per_sm);
+  p.grid = (int)std::min<int64_t>(p.ntiles, (int64_t)h->num_sms * p.ctas);
   p.use = 1;
 }
 
@@ -827,29 +791,62 @@ biofvm_status upload_constants(biofvm *h) {
     if (st) return st;
     if (f32)
       stream_consts_f32(h, axis, t, &c32[(size_t)axis * 2 * h->g.n_sub], h->stream_k0[axis]);
-    // the same inv, mul, pf, pb substrate-major [4][S][npad] for the pipelined kernel
-    auto upload_T = [&](DevBuf &dst) {
-      const int n = axis_len(h, axis), S = h->g.n_sub, npad = pipe_npad_host(n);
-      std::vector<double> tt((size_t)4 * S * npad, 0.0);
-      for (int w = 0; w < 4; w++)
-        for (int i = 0; i < n; i++)
-          for (int s = 0; s < S; s++)
-            tt[((size_t)w * S + s) * npad + i] = t[(size_t)w * n * S + (size_t)i * S + s];
+    // the pipelined kernel's constants as pairs of substrates (pipe_args.h: pipe_tab_pairs)
+    auto upload_T = [&](DevBuf &dst, const PipePlan &q) -> biofvm_status {
+      if (!q.use) return BIOFVM_OK;
+      const int n = axis_len(h, axis), S = h->g.n_sub;
+      const int ncls = pipe_classes(S), cpw = 64 / q.cw, nch = q.W * cpw;
+      const int npad = pipe_npad(nch * q.maxm);
+      std::vector<double> tt((size_t)2 * pipe_tab_pairs(q.maxm, S, q.W, cpw), 0.0);
+      const double *inv = t.data(), *mul = inv + (size_t)n * S;
+      const double *pc = mul + 3 * (size_t)n * S;
+      for (int c = 0; c < ncls; c++)
+        for (int k = 0; k < 2; k++) {  // the pair's substrates
+          const int s = S == 1 ? 0 : ((S % 2 == 0 ? 2 * c : c) + k) % S;
+          auto put = [&](size_t pair, double x) { tt[2 * pair + k] = x; };
+          const double *cfix = pc + (size_t)q.T * S, *in = &c32[(size_t)axis * 2 * S];
+          put((size_t)4 * c, in[s]);
+          put((size_t)4 * c + 1, in[S + s]);
+          put((size_t)4 * c + 2, cfix[s]);
+          put((size_t)4 * c + 3, cfix[S + s]);
+          const size_t p0 = (size_t)4 * ncls;
+          for (int i = 0; i < n; i++) {
+            put(p0 + (size_t)c * npad + i, inv[(size_t)i * S + s]);
+            put(p0 + ((size_t)ncls + c) * npad + i, mul[(size_t)i * S + s]);
+          }
+          const size_t p1 = p0 + (size_t)2 * ncls * npad, p2 = p1 + (size_t)ncls * nch * kWtN;
+          for (int j = 0; j < nch; j++) {
+            const int w = j / cpw;
+            // product over chunks lo..hi within warp w
+            auto prod = [&](int lo, int hi) {
+              double x = 1.0;
+              for (int i = std::max(lo, w * cpw); i <= std::min(hi, (w + 1) * cpw - 1); i++)
+                if (i < q.T) x *= pc[(size_t)i * S + s];
+              return x;
+            };
+            const size_t at = p1 + ((size_t)c * nch + j) * kWtN;
+            put(at + kWtF0, prod(j, j));
+            put(at + kWtF1, prod(j - 1, j));
+            put(at + kWtFx, prod(0, j - 1));
+            put(at + kWtB1, prod(j, j + 1));
+            put(at + kWtBx, prod(j + 1, nch));
+            if (j % cpw == 0) put(p2 + (size_t)c * q.W + w, prod(0, nch));
+          }
+        }
       return upload_doubles(h, dst, tt);
     };
-    if ((st = upload_T(h->tabT[axis])) != BIOFVM_OK) return st;
+    if ((st = upload_T(h->tabT[axis], h->pp[axis])) != BIOFVM_OK) return st;
     if (h->small_use) {  // the small step's own chunk partition
       std::vector<double> ts;
       axis_tables(h, axis, h->small_T[axis], h->small_m[axis], false, ts);
       if ((st = upload_doubles(h, h->small_tab[axis], ts)) != BIOFVM_OK) return st;
     }
-    // the row-padded working copy's plans: tables of their own partition where it differs
+    // the row-padded working copy's plans: tables of their own partition
     const PipePlan &q = h->ppx[axis];
-    h->tabP_own[axis] = h->pitched && (q.T != T || q.m != m);
-    if (h->tabP_own[axis]) {
+    if (h->pitched) {
       axis_tables(h, axis, q.T, q.m, f32, t);
       if ((st = upload_doubles(h, h->tabP[axis], t)) != BIOFVM_OK ||
-          (st = upload_T(h->tabTP[axis])) != BIOFVM_OK)
+          (st = upload_T(h->tabTP[axis], q)) != BIOFVM_OK)
         return st;
     }
   }
@@ -1005,11 +1002,12 @@ cudaError_t launch_pipe(const biofvm *h, int axis, int flags, cudaStream_t st, v
   b.field = field;
   b.stages = p.stages;
   b.stage_elems = p.stage_elems;
-  b.tab = pitched && h->tabP_own[axis]
+  b.tab = pitched
               ? axis_tab_of(h, axis, h->tabP[axis], h->tabTP[axis], p.T, p.m)
               : axis_tab(h, axis);
   b.tab.T = p.T;
   b.tab.m = p.m;
+  b.k0 = h->stream_k0[axis];
   b.flags = flags;
   if (!h->any_dir) b.flags &= ~(kDirBefore | kDirAfter);
   const SrcLists sl = src_lists(h);
@@ -1114,6 +1112,8 @@ cudaError_t launch_x(const biofvm *h, int flags, cudaStream_t st, void *field = 
   a.nz = h->g.nz;
   a.S = h->g.n_sub;
   a.tab = axis_tab(h, 0);
+  a.tab.T = h->xp.T;  // (a stage that does not solve may run here on an axis the pipeline solves)
+  a.tab.m = h->xp.m;
   a.rows_per_cta = h->xp.rows_per_cta;
   a.rows_per_warp = h->xp.rows_per_warp;
   a.warps = h->xp.warps;

@@ -44,9 +44,8 @@ enum : int { kStatusOk = 0, kStatusTimeout = 4 };
 // end (forward) or start (backward) value of chunk u, cw[u][t] being the
 // product of pc over the chunks strictly between u and t.
 //
-// tabT: inv, mul, pf, pb again, substrate-major [4][S][n_pad] with
-// n_pad = 32*ceil(n/32) + 1 (the layout the pipelined kernel stages into
-// shared memory; the planner takes that kernel only when they fit).
+// tabT: the pipelined kernel's constants (pipe_args.h), which it stages into
+// shared memory.
 struct AxisTab {
   const void *inv, *mul, *pf, *pb, *pc, *cfix, *cw, *tabT;
   int n, T, m;
@@ -225,8 +224,7 @@ cudaError_t launch_batch_f64(const BatchArgs &a, int maxm, int grid, cudaStream_
 cudaError_t launch_batch_f32(const BatchArgs &a, int maxm, int grid, cudaStream_t st);
 cudaError_t batch_occupancy_f64(int maxm, int *out);
 cudaError_t batch_occupancy_f32(int maxm, int *out);
-// The same sweep for fields stored in 16 bits (bf16 / fp16), FP32 arithmetic;
-// chunk capacities 32 and 64.
+// The same sweep for fields stored in 16 bits (bf16 / fp16), FP32 arithmetic.
 cudaError_t allow_pipe_smem_bf16(int maxm, size_t bytes);
 cudaError_t allow_pipe_smem_fp16(int maxm, size_t bytes);
 cudaError_t launch_pipe_bf16(const CUtensorMap &map, const PipeArgs &a, int maxm, int grid,
@@ -238,10 +236,4 @@ cudaError_t launch_pipe_fp16(const CUtensorMap &map, const PipeArgs &a, int maxm
 // of a field whose rows are not 16-byte multiples).
 cudaError_t launch_pitch_rows(const void *src, void *dst, int64_t rows, int len, int spitch,
                               int dpitch, size_t esz, int grid, cudaStream_t st);
-// Largest CTA the FP32 pipelined sweep with chunk capacity maxm may use.
-int pipe_max_threads_f32(int maxm);
-// Substrate-major constants of the pipelined sweep (elements): [4][S][npad].
-inline int pipe_npad_host(int n) { return (n + 31) / 32 * 32 + 1; }
-inline int pipe_tab_elems_host(int n, int S) { return 4 * S * pipe_npad_host(n); }
-
 }  // namespace bfv

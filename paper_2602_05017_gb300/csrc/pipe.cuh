@@ -1,11 +1,10 @@
 // Persistent, TMA-pipelined sweep kernel for sm_103a (x, y and z sweeps).
 //
-// Same arithmetic as the plain kernels of sweeps.cuh -- partitioned Thomas of
-// Algorithm 1 on the App. A system, FP32 in defect-correction form -- but
-// every tile of CW independent lines ("columns") x n positions moves through
-// a ring of shared-memory stages.  CW = 32 normally; for lines so long that two
-// stages of 32 columns do not fit in shared memory, tiles of CW = 16 columns,
-// and each consumer warp then solves two chunks, one per half-warp:
+// The arithmetic is the plain kernels' of sweeps.cuh -- partitioned Thomas of
+// Algorithm 1 on the App. A system, FP32 in defect-correction form -- on tiles
+// of CW independent lines ("columns") x n positions that move through a ring
+// of shared-memory stages.  CW = 32 normally; 16 for lines so long that two
+// stages of 32 columns do not fit:
 //
 //   warp 0 (producer): TMA loads of tile k+NS-1 (cp.async.bulk.tensor boxes
 //     for y/z tiles, issued by lane 0; one cp.async.bulk per row for x tiles,
@@ -18,14 +17,27 @@
 //     has landed -- running ahead of the consumers, who solve earlier tiles --
 //     and arrives on mbarrier `ready`, which the consumers then wait for
 //     instead of `full`;
-//   the next ceil(T*CW/32) warps (consumers): chunk t of every column of the staged
-//     tile, in registers (thread (warp w, lane l): chunk (w-1)*32/CW + l/CW of
-//     column l % CW).  Halos and chunk carries cross warps through shared memory
+//   the next W warps (consumers): each thread holds one chunk (MAXM positions)
+//     of a PAIR of columns in registers and works on both with packed FP32
+//     instructions; a warp holds 64/CW chunks of the tile's CW/2 pairs.
+//     Carries cross a warp by shuffles and the CTA through shared memory,
 //     between two named barriers per tile that only consumers join.
 //
+// What bounds it.  One column per thread, coefficients and carry weights read
+// from shared memory at every position and a guard on every ragged position
+// took 27 issued instructions per element and left the sweep waiting on them:
+// 0.51 ms a sweep at 400^3 x 4 (4.0 TB/s).  Pairs halve the instructions,
+// chunks whose coefficients have reached their interior values (all but the
+// first one or two and the last of a line) read none, and running the
+// recurrences again from the true carry replaces the correction passes: about
+// six instructions per element.  Chunks are short (16 positions) because the
+// four dependent chains per tile are the remaining latency.  Measured, x / y /
+// z of 400^3 x 4: 0.540 / 0.506 / 0.513 ms before, 0.34 / 0.33 / 0.39 after
+// (HBM copy rate: 0.306); the z sweep's rows are 128 bytes, a plane apart.
+//
 // The grid is persistent (tiles strided by gridDim.x), so loads of later
-// tiles overlap the solve and the store of earlier ones.  The axis constants
-// and the carry weights are staged once per CTA.
+// tiles overlap the solve and the store of earlier ones.  The constants are
+// staged once per CTA.
 //
 // Every mbarrier wait is bounded (mbar_wait_bounded): on a timeout the status
 // word is set, the consumers agree to stop at the first carry barrier, which
@@ -103,122 +115,332 @@ __device__ __forceinline__ bool consumers_all(bool ok, int nthreads) {
   return r != 0;
 }
 
-template <typename E, int MAXM>
-struct PipeBound {  // chunk registers + about 96 for addressing, carries, constants
-  static constexpr int regs = MAXM * (int)sizeof(E) / 4 + 96;
-  static constexpr int raw = 65536 / regs;
-  static constexpr int threads = (raw >= 1024 ? 1024 : raw) / 32 * 32;
+// Two FP32 values in one 64-bit register pair: every arithmetic instruction of
+// the solve works on two columns at once (fma.rn.f32x2 and friends, sm_100+;
+// each half rounds as the scalar instruction would).
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 f2_pack(float x, float y) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ float2 f2_unpack(f2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+  f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
+  f2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// A thread's two columns of a staged tile, positions ps elements apart.
+//   PAIR: the columns are neighbours (c, c + 1) at an even offset: one access
+//         of two elements per position;
+//   VEC > 1: VEC consecutive positions arrive in one access per column
+//         (x tiles of one substrate: the two columns are rows) or for the pair
+//         (x tiles of two);
+//   otherwise two scalar accesses per position.
+template <typename H, int PS, bool PAIR, int VEC>
+struct ColPair {
+  H *p0, *p1;  // position 0 of the thread's chunk in either column (PAIR: p1 unused)
+  int ps_rt;
+  __device__ __forceinline__ int ps() const { return PS > 0 ? PS : ps_rt; }
+  __device__ __forceinline__ f2 one(int i) const {  // any position
+    if constexpr (PAIR) {
+      return load2(p0 + i * ps());
+    } else {
+      return f2_pack(widen<float>(p0[i * ps()]), widen<float>(p1[i * ps()]));
+    }
+  }
+  __device__ __forceinline__ void put(int i, f2 v, bool st0, bool st1) const {
+    if constexpr (PAIR) {  // (both columns are in the tile: st0 == st1)
+      if (st0) store2(p0 + i * ps(), v);
+    } else {
+      const float2 x = f2_unpack(v);
+      if (st0) p0[i * ps()] = narrow<H>(x.x);
+      if (st1) p1[i * ps()] = narrow<H>(x.y);
+    }
+  }
+  // positions i .. i+VEC-1, i a multiple of VEC (and the chunk start too)
+  __device__ __forceinline__ void block(int i, f2 (&d)[VEC]) const {
+    if constexpr (VEC == 1) {
+      d[0] = one(i);
+    } else if constexpr (PAIR) {  // PS == 2, VEC == 2
+      float x[4];
+      load4(p0 + i * 2, x);
+      d[0] = f2_pack(x[0], x[1]);
+      d[1] = f2_pack(x[2], x[3]);
+    } else {  // PS == 1, VEC == 4
+      float x[4], y[4];
+      load4(p0 + i, x);
+      load4(p1 + i, y);
+#pragma unroll
+      for (int k = 0; k < 4; k++) d[k] = f2_pack(x[k], y[k]);
+    }
+  }
+  __device__ __forceinline__ void put_block(int i, const f2 (&d)[VEC], bool st0, bool st1) const {
+    if constexpr (VEC == 1) {
+      put(i, d[0], st0, st1);
+    } else if constexpr (PAIR) {
+      const float2 a = f2_unpack(d[0]), b = f2_unpack(d[1]);
+      store4(p0 + i * 2, a.x, a.y, b.x, b.y);
+    } else {
+      float2 a[4];
+#pragma unroll
+      for (int k = 0; k < 4; k++) a[k] = f2_unpack(d[k]);
+      store4(p0 + i, a[0].x, a[1].x, a[2].x, a[3].x);
+      store4(p1 + i, a[0].y, a[1].y, a[2].y, a[3].y);
+    }
+  }
+
+ private:
+  static __device__ __forceinline__ f2 load2(const H *q) {
+    if constexpr (std::is_same<H, float>::value) {
+      return *reinterpret_cast<const f2 *>(q);
+    } else if constexpr (std::is_same<H, __half>::value) {
+      const float2 v = __half22float2(*reinterpret_cast<const __half2 *>(q));
+      return f2_pack(v.x, v.y);
+    } else {
+      const float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(q));
+      return f2_pack(v.x, v.y);
+    }
+  }
+  static __device__ __forceinline__ void store2(H *q, f2 v) {
+    if constexpr (std::is_same<H, float>::value) {
+      *reinterpret_cast<f2 *>(q) = v;
+    } else if constexpr (std::is_same<H, __half>::value) {
+      const float2 x = f2_unpack(v);
+      *reinterpret_cast<__half2 *>(q) = __floats2half2_rn(x.x, x.y);
+    } else {
+      const float2 x = f2_unpack(v);
+      *reinterpret_cast<__nv_bfloat162 *>(q) = __floats2bfloat162_rn(x.x, x.y);
+    }
+  }
+  static __device__ __forceinline__ void load4(const H *q, float (&x)[4]) {
+    if constexpr (std::is_same<H, float>::value) {
+      const float4 v = *reinterpret_cast<const float4 *>(q);
+      x[0] = v.x, x[1] = v.y, x[2] = v.z, x[3] = v.w;
+    } else {
+      const uint2 v = *reinterpret_cast<const uint2 *>(q);
+      H h[4];
+      memcpy(h, &v, 8);
+#pragma unroll
+      for (int k = 0; k < 4; k++) x[k] = widen<float>(h[k]);
+    }
+  }
+  static __device__ __forceinline__ void store4(H *q, float a, float b, float c, float d) {
+    if constexpr (std::is_same<H, float>::value) {
+      *reinterpret_cast<float4 *>(q) = make_float4(a, b, c, d);
+    } else {
+      const H h[4] = {narrow<H>(a), narrow<H>(b), narrow<H>(c), narrow<H>(d)};
+      uint2 v;
+      memcpy(&v, h, 8);
+      *reinterpret_cast<uint2 *>(q) = v;
+    }
+  }
 };
 
-// Constants of the pipelined kernel: inv, mul, pf, pb substrate-major
-// [S][n_pad] (n_pad = 1 mod 32, so lanes of different substrates read
-// different banks and each thread walks its own row with compile-time
-// offsets) -- AxisTab::tabT, copied into shared memory (the planner only
-// takes this kernel when they fit).
-__host__ __device__ inline int pipe_npad(int n) { return (n + 31) / 32 * 32 + 1; }
+// A chunk pair's constants in shared memory (pipe_args.h).
+struct PairCoef {
+  const f2 *K;                // interior inv' and mul; c_hi, c_lo
+  const ulonglong2 *Ti, *Tm;  // inv' and mul of the chunk's positions, two at a time (0 past the
+                              // line's end)
+  const f2 *wt;               // the chunk's carry weights (kWt*)
+  const f2 *pw;               // [W] products of mul over each warp's chunks
+};
+// What a thread does with the Dirichlet application after the solve.
+struct PairDir {
+  bool on0, on1;    // the column's substrate is flagged
+  bool face0, face1;  // the whole line lies on a face
+  bool any;         // some lane of the warp has a flagged column
+  float val0, val1;
+};
 
-// One chunk of one column: e = L_N d (FP32), forward elimination, carry in,
-// back substitution, carry in, c d + y (FP32), Dirichlet, write-back.
-// FULL: the chunk has exactly MAXM positions (no per-position guards).
-// PS > 0: compile-time stride between positions in the staged tile.
-template <typename E, int MAXM, bool FULL, int PS, int CW, typename H>
-__device__ __forceinline__ bool pipe_chunk(H *p, const int ps_rt, const int len, const int lo,
-                                           const int n, const int t, const int T, const int c,
-                                           const E *Ti, const E *Tm, const E *Tf, const E *Tb,
-                                           const E *Tcw, const int S, const int s, const E chi,
-                                           const E clo, E *s_end, E *s_beg, const int ncons,
-                                           const bool dir, const bool face, const E dval,
-                                           const bool ok) {
-  const int ps = PS > 0 ? PS : ps_rt;
-  E v[MAXM];
+// Chunk q of a warp (lanes q*PW ..) ends with B_q from a zero carry; the inclusive
+// scan over the warp's chunks gives the end value of chunks 0..q, and the last
+// one is the warp's.  The suffix scan serves the back substitution.
+template <int CPW>
+__device__ __forceinline__ f2 scan_fwd(f2 B, int q, const f2 *wt) {
+  constexpr int PW = 32 / CPW;
 #pragma unroll
-  for (int i = 0; i < MAXM; i++)
-    if (FULL || i < len) v[i] = widen<E>(p[i * ps]);
-  if constexpr (kDefect<E>) {
-    // e = L_N d.  At the two ends of the line the zero-flux rows equal the
-    // interior formula with a mirrored ghost value (d_{-1} = d_0,
-    // d_n = d_{n-1}), so no position needs a branch.
-    E prev = E(0), after = E(0);
-    if (len > 0) {
-      prev = lo > 0 ? widen<E>(p[-ps]) : v[0];
-      // (the last value is re-read from the tile: selecting v[len-1] would
-      // index the register array dynamically)
-      const E last = FULL ? v[MAXM - 1] : widen<E>(p[(len - 1) * ps]);
-      after = lo + len < n ? widen<E>(p[(FULL ? MAXM : len) * ps]) : last;
-    }
-#pragma unroll
-    for (int i = 0; i < MAXM; i++)
-      if (FULL || i < len) {
-        const E cur = v[i];
-        const E nxt = (i + 1 < MAXM && (FULL || i + 1 < len)) ? v[i + 1] : after;
-        v[i] = (cur - prev) + (cur - nxt);
-        prev = cur;
-      }
+  for (int d = 1, k = kWtF0; d < CPW; d <<= 1, k++) {
+    const f2 B2 = __shfl_up_sync(0xffffffffu, B, d * PW);
+    if (q >= d) B = f2_fma(wt[k], B2, B);
   }
-  E g = E(0);
+  return B;
+}
+template <int CPW>
+__device__ __forceinline__ f2 scan_bwd(f2 B, int q, const f2 *wt) {
+  constexpr int PW = 32 / CPW;
 #pragma unroll
-  for (int i = 0; i < MAXM; i++)
-    if (FULL || i < len) {
-      g = fma(Tm[i], g, v[i] * Ti[i]);
-      v[i] = g;
+  for (int d = 1; d < CPW; d <<= 1) {
+    const f2 B2 = __shfl_down_sync(0xffffffffu, B, d * PW);
+    if (q + d < CPW) B = f2_fma(wt[d == 1 ? kWtF0 : kWtB1], B2, B);
+  }
+  return B;
+}
+
+// One chunk of a column pair: e = L_N d, forward recurrence from a zero carry
+// (its end only), the true carry, the forward recurrence again (kept), the same
+// backward, c d + y, Dirichlet, write-back.  Running each recurrence a second
+// time from the true carry costs one packed FMA per position -- the products
+// pf, pb that would correct the first result cost the same FMA and a
+// shared-memory load each.
+// FAST: MAXM positions of constant coefficients strictly inside the line.
+// Returns false when a consumer's wait for the tile timed out.
+template <int MAXM, bool FAST, int CPW, int VEC, typename Cols>
+__device__ __forceinline__ bool pipe_chunk(const Cols col, const int len, const int lo,
+                                           const int n, const int wc, const int W, const int q,
+                                           const int p, const PairCoef &cf, f2 *s_end,
+                                           f2 *s_beg, const int ncons, const PairDir &dir,
+                                           const bool st0, const bool st1, const bool ok) {
+  constexpr int PW = 32 / CPW;
+  const unsigned FULL = 0xffffffffu;
+  f2 v[MAXM];
+  const f2 zero = 0;
+  f2 g = zero;
+  auto at = [&](int i) { return col.one(max(-lo, min(i, n - 1 - lo))); };  // position clamped
+  if constexpr (FAST) {
+    const f2 c0 = cf.K[0], c1 = cf.K[1];
+    const f2 before = col.one(-1), after = col.one(MAXM);
+#pragma unroll
+    for (int i = 0; i < MAXM; i += VEC) {
+      f2 b[VEC];
+      col.block(i, b);
+#pragma unroll
+      for (int k = 0; k < VEC; k++) v[i + k] = b[k];
     }
-  s_end[t * CW + c] = g;
+    f2 am = f2_sub(before, v[0]);  // d_{i-1} - d_i
+#pragma unroll
+    for (int i = 0; i < MAXM; i++) {
+      const f2 a = f2_sub(v[i], i + 1 < MAXM ? v[i + 1] : after);
+      v[i] = f2_mul(f2_sub(a, am), c0);  // (d_i - d_{i-1}) + (d_i - d_{i+1})
+      am = a;
+      g = f2_fma(c1, g, v[i]);
+    }
+  } else {
+    // Positions are clamped to the line: the ghost values d_{-1} = d_0 and d_n = d_{n-1} of the
+    // zero-flux ends come of themselves, and what follows the line's end has zero differences
+    // and zero coefficients, so that it carries nothing into the line from either side.
+#pragma unroll
+    for (int i = 0; i < MAXM; i++) v[i] = at(i);
+    f2 am = f2_sub(at(-1), v[0]);
+    const f2 after = at(MAXM);
+#pragma unroll
+    for (int i = 0; i < MAXM; i += 2) {
+      const ulonglong2 ti = cf.Ti[i / 2], tm = cf.Tm[i / 2];
+#pragma unroll
+      for (int k = i; k < i + 2; k++) {
+        const f2 a = f2_sub(v[k], k + 1 < MAXM ? v[k + 1] : after);
+        v[k] = f2_mul(f2_sub(a, am), k == i ? ti.x : ti.y);
+        am = a;
+        g = f2_fma(k == i ? tm.x : tm.y, g, v[k]);
+      }
+    }
+  }
+  g = scan_fwd<CPW>(g, q, cf.wt);
+  if (q == CPW - 1) s_end[wc * PW + p] = g;
+  f2 prev = __shfl_up_sync(FULL, g, PW);
   // The first carry barrier also ANDs the outcome of every consumer's wait
   // for the tile: on a timeout all consumers leave together, before any
   // write-back (what they computed from the unfinished stage stays local).
   if (!consumers_all(ok, ncons)) return false;
-  // carry weights Tcw[(u*T + t)*S + s] walked with pointer steps (no index
-  // arithmetic per term), in the same order as the closed form's sum; not
-  // unrolled (unrolling by 4 measured 5% slower on the y/z tiles)
-  const int dw = T * S;
-  if (t > 0 && t < T) {  // chunk 0 enters with a zero carry (t == T: a half-warp with no chunk)
-    E carry = E(0);
-    const E *w = Tcw + ((t - 1) * T + t) * S + s;
-    const E *q = s_end + (t - 1) * CW + c;
-#pragma unroll 1
-    for (int u = t - 1; u >= 0; u--, w -= dw, q -= CW) carry = fma(*w, *q, carry);
-#pragma unroll
-    for (int i = 0; i < MAXM; i++)
-      if (FULL || i < len) v[i] = fma(Tf[i], carry, v[i]);
+  {
+    f2 c = zero;  // what the warps before this one carry in
+#pragma unroll 4
+    for (int u = 0; u < wc; u++) c = f2_fma(cf.pw[u], c, s_end[u * PW + p]);
+    g = q == 0 ? c : f2_fma(cf.wt[kWtFx], c, prev);
   }
-  E x = E(0);
+  f2 x = zero;
+  if constexpr (FAST) {
+    const f2 c1 = cf.K[1];
 #pragma unroll
-  for (int i = MAXM - 1; i >= 0; i--)
-    if (FULL || i < len) {
-      x = fma(Tm[i], x, v[i]);
-      v[i] = x;
+    for (int i = 0; i < MAXM; i++) {
+      g = f2_fma(c1, g, v[i]);
+      v[i] = g;
     }
-  s_beg[t * CW + c] = x;
+#pragma unroll
+    for (int i = MAXM - 1; i >= 0; i--) x = f2_fma(c1, x, v[i]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < MAXM; i += 2) {
+      const ulonglong2 tm = cf.Tm[i / 2];
+      v[i] = f2_fma(tm.x, g, v[i]);
+      g = v[i + 1] = f2_fma(tm.y, v[i], v[i + 1]);
+    }
+#pragma unroll
+    for (int i = MAXM - 2; i >= 0; i -= 2) {
+      const ulonglong2 tm = cf.Tm[i / 2];
+      x = f2_fma(tm.x, f2_fma(tm.y, x, v[i + 1]), v[i]);
+    }
+  }
+  x = scan_bwd<CPW>(x, q, cf.wt);
+  if (q == 0) s_beg[wc * PW + p] = x;
+  prev = __shfl_down_sync(FULL, x, PW);
   consumers_sync(ncons);
-  if (t + 1 < T) {  // the last chunk enters with a zero carry
-    E carry = E(0);
-    const E *w = Tcw + ((t + 1) * T + t) * S + s;
-    const E *q = s_beg + (t + 1) * CW + c;
-#pragma unroll 1
-    for (int u = t + 1; u < T; u++, w += dw, q += CW) carry = fma(*w, *q, carry);
-#pragma unroll
-    for (int i = 0; i < MAXM; i++)
-      if (FULL || i < len) v[i] = fma(Tb[i], carry, v[i]);
-  }
-  if constexpr (kDefect<E>) {  // x = c_hi d + (c_lo d + y), d from the staged tile
-#pragma unroll
-    for (int i = 0; i < MAXM; i++)
-      if (FULL || i < len) {
-        const E d = widen<E>(p[i * ps]);
-        v[i] = fma(chi, d, fma(clo, d, v[i]));
-      }
-  }
-  if (dir && len > 0) {
-#pragma unroll
-    for (int i = 0; i < MAXM; i++)
-      if ((FULL || i < len) && (face || lo + i == 0 || lo + i == n - 1)) v[i] = dval;
+  {
+    f2 c = zero;
+#pragma unroll 4
+    for (int u = W - 1; u > wc; u--) c = f2_fma(cf.pw[u], c, s_beg[u * PW + p]);
+    x = q == CPW - 1 ? c : f2_fma(cf.wt[kWtBx], c, prev);
   }
   // No barrier before the write-back: the only reads of other chunks' positions
   // (the halos of e = L_N d) happen before the first barrier above, and the
   // carry arrays are rewritten only after barriers every warp has passed.
+  const f2 chi = cf.K[2], clo = cf.K[3];
+  auto with_dir = [&](f2 r, bool end) {
+    float2 a = f2_unpack(r);
+    if (dir.on0 && (dir.face0 || end)) a.x = dir.val0;
+    if (dir.on1 && (dir.face1 || end)) a.y = dir.val1;
+    return f2_pack(a.x, a.y);
+  };
+  if constexpr (FAST) {
+    const f2 c1 = cf.K[1];
+    auto finish = [&](auto dirc) {
 #pragma unroll
-  for (int i = 0; i < MAXM; i++)
-    if (FULL || i < len) p[i * ps] = narrow<H>(v[i]);
+      for (int i = MAXM - VEC; i >= 0; i -= VEC) {
+        f2 d[VEC];
+        col.block(i, d);
+#pragma unroll
+        for (int k = VEC - 1; k >= 0; k--) {
+          x = f2_fma(c1, x, v[i + k]);
+          d[k] = f2_fma(chi, d[k], f2_fma(clo, d[k], x));  // c_hi d + (c_lo d + y)
+          if constexpr (decltype(dirc)::value) d[k] = with_dir(d[k], false);
+        }
+        col.put_block(i, d, st0, st1);
+      }
+    };
+    if (dir.any) finish(std::true_type{}); else finish(std::false_type{});
+  } else {
+    auto finish = [&](auto dirc) {
+#pragma unroll
+      for (int i = MAXM - 2; i >= 0; i -= 2) {
+        const ulonglong2 tm = cf.Tm[i / 2];
+#pragma unroll
+        for (int k = i + 1; k >= i; k--) {
+          x = f2_fma(k == i ? tm.x : tm.y, x, v[k]);
+          const f2 d = at(k);
+          f2 r = f2_fma(chi, d, f2_fma(clo, d, x));
+          if constexpr (decltype(dirc)::value)
+            r = with_dir(r, lo + k == 0 || lo + k == n - 1);
+          col.put(k, r, st0 && k < len, st1 && k < len);
+        }
+      }
+    };
+    if (dir.any) finish(std::true_type{}); else finish(std::false_type{});
+  }
   return true;
 }
 
@@ -228,53 +450,51 @@ __device__ __forceinline__ bool pipe_chunk(H *p, const int ps_rt, const int len,
 // per-access address arithmetic; 0: S read at run time.  CW: columns per tile
 // (32, or 16 for long lines).  H: the field's storage type (E, or bf16 / fp16
 // with E = float): stages and TMA copies hold H, registers and constants E.
-template <typename E, int MAXM, int MODE, int PSX = 0, int CW = 32, typename H = E>
-__global__ void __launch_bounds__(PipeBound<E, MAXM>::threads)
+template <int MAXM, int MODE, int PSX = 0, int CW = 32, typename H = float>
+__global__ void __maxnreg__(pipe_regs(MAXM))
     sweep_pipe_kernel(const __grid_constant__ CUtensorMap map, const PipeArgs a) {
   static_assert(CW == 32 || CW == 16, "tiles of 32 or 16 columns");
-  constexpr int CPW = 32 / CW;  // chunks per consumer warp
-  extern __shared__ __align__(1024) unsigned char smem_raw[];
-  const int T = a.tab.T, m = a.tab.m, n = a.n, S = a.S, NS = a.stages;
+  typedef float E;
+  constexpr int CPW = 64 / CW;    // chunks per consumer warp
+  constexpr int PW = 32 / CPW;    // column pairs of the tile
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int T = a.tab.T, n = a.n, S = a.S, NS = a.stages;
   const int64_t stage_elems = a.stage_elems;
-  const int npad = pipe_npad(n);
-  H *stage0 = reinterpret_cast<H *>(smem_raw);
-  // [4][S][npad], 16-byte aligned after the stages: offset arithmetic on the shared array itself
-  // (a pointer rounded through an integer would hide from the compiler that the constants and
-  // carry arrays derived from it live in shared memory, turning their loads into generic ones)
-  E *tab = reinterpret_cast<E *>(smem_raw + ((size_t)NS * stage_elems * sizeof(H) + 15) / 16 * 16);
   const int W = (T + CPW - 1) / CPW;  // consumer warps
-  E *s_end = tab + 4 * S * npad;      // [W*32]: chunk t, column c at t*CW + c
-  E *s_beg = s_end + W * 32;
-  E *s_cw = s_beg + W * 32;  // [T][T][S] carry weights
-  uint64_t *full = reinterpret_cast<uint64_t *>(
-      (reinterpret_cast<uintptr_t>(s_cw + T * T * S) + 15) & ~uintptr_t(15));
+  const int ncls = pipe_classes(S), npad = pipe_npad(W * CPW * MAXM);
+  H *stage0 = reinterpret_cast<H *>(smem_raw);
+  // constants (pipe_tab_pairs), 16-byte aligned after the stages: offset arithmetic on the shared
+  // array itself (a pointer rounded through an integer would hide from the compiler that what is
+  // derived from it lives in shared memory, turning its loads into generic ones)
+  f2 *tab = reinterpret_cast<f2 *>(smem_raw + ((size_t)NS * stage_elems * sizeof(H) + 15) / 16 * 16);
+  const int ntab = pipe_tab_pairs(MAXM, S, W, CPW);
+  f2 *s_end = tab + ntab;   // [W][PW] warp ends (forward)
+  f2 *s_beg = s_end + W * PW;  // [W][PW] warp starts (backward)
+  uint64_t *full = reinterpret_cast<uint64_t *>(s_beg + W * PW);
   uint64_t *done = full + NS;
   uint64_t *ready = done + NS;  // x tiles with a preparation: the stage is prepared
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long first = blockIdx.x;
-  const long long count = (a.ntiles - first + gridDim.x - 1) / gridDim.x;
+  // (the planner keeps tile, row and column counts below 2^31)
+  const int first = blockIdx.x;
+  const int count = ((int)a.ntiles - first + (int)gridDim.x - 1) / (int)gridDim.x;
   const int ncons = W * 32;
   H *field = static_cast<H *>(a.field);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; s++) {
       mbar_init(&full[s], 1);
-      mbar_init(&done[s], ncons);
+      mbar_init(&done[s], W);
       mbar_init(&ready[s], 1);
     }
     fence_mbar_init();
     fence_proxy_async_smem();
   }
   {
-    const E *gT = static_cast<const E *>(a.tab.tabT);
-    for (int q = threadIdx.x; q < 4 * S * npad; q += blockDim.x) tab[q] = __ldg(gT + q);
-    const E *gW = static_cast<const E *>(a.tab.cw);
-    for (int q = threadIdx.x; q < T * T * S; q += blockDim.x) s_cw[q] = __ldg(gW + q);
+    const f2 *gT = static_cast<const f2 *>(a.tab.tabT);
+    for (int q = threadIdx.x; q < ntab; q += blockDim.x) tab[q] = __ldg(gT + q);
   }
   __syncthreads();
-  const E *s_inv = tab, *s_mul = tab + S * npad, *s_pf = s_mul + S * npad, *s_pb = s_pf + S * npad;
-  const E *g_cfix = static_cast<const E *>(a.tab.cfix);
 
   // x tiles: Src and B before the solve, applied by warp 1 (the preparer) when
   // the launch has one (a.prep_warp: the host sets it exactly when there is a
@@ -465,42 +685,73 @@ __global__ void __launch_bounds__(PipeBound<E, MAXM>::threads)
   }
 
   // ---------------------------------------------------------------- consumers
-  const int wc = warp - cons0;                     // consumer warp
-  const int c = CW == 32 ? lane : (lane & (CW - 1));  // column of the tile
-  const int t = wc * CPW + lane / CW;              // chunk (t == T: no chunk)
-  const int lo = t * m;
-  const int len_full = t < T ? min(m, n - lo) : 0;
-  const int colbase = MODE == 0 ? (c / S) * a.pitch + c % S : c;
-  const int ps_rt = MODE == 0 ? S : CW;
-  const E *Tcw = s_cw;  // [T][T][S], staged beside the other constants
+  const int wc = warp - cons0;          // consumer warp
+  const int p = lane % PW, q = lane / PW;  // column pair, chunk of the warp
+  const int t = wc * CPW + q;              // chunk (t >= T: none)
+  // x tiles of one substrate pair row p with row p + PW (consecutive lanes then read
+  // consecutive rows, whose 16-byte accesses hit distinct banks); all others pair neighbours
+  constexpr bool kRowPairs = MODE == 0 && PSX == 1;
+  const int col0 = kRowPairs ? p : 2 * p, col1 = kRowPairs ? p + PW : 2 * p + 1;
+  const int lo = t * MAXM;
+  const int len = max(0, min(MAXM, n - lo));  // (0: a lane without a chunk)
+  // columns of the stage: an x tile of rows_per_tile * S < CW columns leaves lanes without one,
+  // which work on column 0 and store nothing
+  const int ncol = MODE == 0 ? a.rows_per_tile * S : CW;
+  const bool st0 = col0 < ncol, st1 = col1 < ncol;
+  auto offset = [&](int c) {
+    if (c >= ncol) c = 0;
+    return MODE == 0 ? (c / S) * a.pitch + c % S : c;
+  };
+  constexpr int PS = MODE == 0 ? PSX : CW;
+  constexpr bool kPair = PS > 0 && PS % 2 == 0;
+  constexpr int VEC = MODE != 0 ? 1 : PSX == 1 ? 4 : PSX == 2 ? 2 : 1;
+  ColPair<H, PS, kPair, VEC> col;
+  col.ps_rt = MODE == 0 ? S : CW;
+  const int off0 = offset(col0) + lo * col.ps(), off1 = offset(col1) + lo * col.ps();
+  // constant coefficients strictly inside the line, for the whole warp
+  const bool fast = __all_sync(0xffffffffu, len == MAXM && lo >= max(a.k0, 1) && lo + MAXM <= n - 1);
   const bool dir_after = (a.flags & kDirAfter) != 0;
   const int ctid = threadIdx.x - 32 * cons0;  // consumer thread
   long long cn0 = 0, cn1 = 0;                 // entry range of the next tile (dense check)
   if (srcs) tile_range(0, cn0, cn1);
-  // A thread's substrate is the same in every tile when S divides the tile width (and, for
+  PairCoef cf;
+  PairDir dir;
+  auto set_substrates = [&](int sa, int sb) {
+    const int cls = S == 1 ? 0 : S % 2 == 0 ? sa / 2 : sa;
+    cf.K = tab + cls * 4;
+    cf.Ti = reinterpret_cast<const ulonglong2 *>(tab + 4 * ncls + cls * npad + lo);
+    cf.Tm = reinterpret_cast<const ulonglong2 *>(tab + 4 * ncls + (ncls + cls) * npad + lo);
+    const f2 *w = tab + 4 * ncls + 2 * ncls * npad;
+    cf.wt = w + (cls * (W * CPW) + t) * kWtN;
+    cf.pw = w + ncls * (W * CPW) * kWtN + cls * W;
+    dir.on0 = dir_after && a.dir_on[sa];
+    dir.on1 = dir_after && a.dir_on[sb];
+    dir.val0 = dir.on0 ? dir_value<E>(a.flags, a.dir_val, sa) : E(0);
+    dir.val1 = dir.on1 ? dir_value<E>(a.flags, a.dir_val, sb) : E(0);
+    dir.face0 = dir.face1 = false;
+    dir.any = __any_sync(0xffffffffu, dir.on0 || dir.on1);
+  };
+  // A thread's substrates are the same in every tile when S divides the tile width (and, for
   // z tiles, the row pitch): its per-substrate constants are then loaded once, not per tile.
   const bool s_fixed = MODE == 0 || (CW % S == 0 && (a.mode == 1 || a.gpitch % S == 0));
-  const int sf = c % S;
-  const E chi_f = s_fixed ? __ldg(g_cfix + sf) : E(0), clo_f = s_fixed ? __ldg(g_cfix + S + sf) : E(0);
-  const bool dir_f = s_fixed && dir_after && a.dir_on[sf];
-  const E dval_f = dir_f ? dir_value<E>(a.flags, a.dir_val, sf) : E(0);
-  // The planner keeps tile, row and column counts below 2^31, so the per-tile
-  // index arithmetic below runs in 32 bits (a 64-bit division is a long
+  if (s_fixed) set_substrates(col0 % S, col1 % S);
+  // The per-tile index arithmetic runs in 32 bits (a 64-bit division is a long
   // software sequence, and every consumer thread repeats it per tile).
-  for (long long k = 0; k < count; k++) {
-    const int st = (int)(k % NS);
+  int st = -1, round = -1;  // the tile's stage, how often the ring has wrapped
+  for (int k = 0; k < count; k++) {
+    if (++st == NS) st = 0;
+    if (st == 0) round++;
     // (a timed-out wait is acted on at the first carry barrier of the chunk
     // solve; the steps before it only touch this stage and registers)
     // (x tiles with a preparation: the preparer's `ready`, after its own wait for the data)
-    const bool ok = mbar_wait_bounded(prep ? &ready[st] : &full[st], (uint32_t)((k / NS) & 1),
-                                      a.status);
-    const long long tile = first + k * gridDim.x;
+    const bool ok = mbar_wait_bounded(prep ? &ready[st] : &full[st], (uint32_t)(round & 1), a.status);
+    const int tile = first + k * (int)gridDim.x;
     H *const stg = stage0 + st * stage_elems;
     if (srcs) {
       const long long c0 = cn0, c1 = cn1;
       tile_range(k + 1, cn0, cn1);  // the next tile's range, used one tile later
       if (is_dense(c0, c1)) {       // every consumer agrees (global data); done whatever `ok`
-        const long long r0 = tile * a.rows_per_tile;
+        const long long r0 = (long long)tile * a.rows_per_tile;
         const int rows = (int)min((long long)a.rows_per_tile, a.nrows - r0);
         constexpr int U = 4;
         for (long long eb = c0 + ctid; eb < c1; eb += (long long)ncons * U) {
@@ -528,145 +779,106 @@ __global__ void __launch_bounds__(PipeBound<E, MAXM>::threads)
         }
       }
     }
-    int s;
-    bool active, face = false;
     if constexpr (MODE == 0) {
-      const long long r0 = tile * a.rows_per_tile;
-      const int rows = (int)min((long long)a.rows_per_tile, a.nrows - r0);
-      s = c % S;
-      active = c < a.rows_per_tile * S && c / S < rows;
-      if (dir_after) {  // (only the Dirichlet application after the solve needs the face)
-        const uint32_t row = (uint32_t)r0 + (uint32_t)(c / S);
-        const int z = (int)(row / (uint32_t)a.ny), y = (int)row - z * a.ny;
-        face = y == 0 || y == a.ny - 1 || z == 0 || z == a.nz - 1;
+      if (dir.any) {  // (only the Dirichlet application after the solve needs the face)
+        const uint32_t r0 = (uint32_t)(tile * a.rows_per_tile);
+        auto face = [&](int c) {
+          const uint32_t row = r0 + (uint32_t)(c / S);
+          const int z = (int)(row / (uint32_t)a.ny), y = (int)row - z * a.ny;
+          return y == 0 || y == a.ny - 1 || z == 0 || z == a.nz - 1;
+        };
+        dir.face0 = face(col0);
+        dir.face1 = kRowPairs || PSX == 0 ? face(col1) : dir.face0;
       }
     } else {
+      // columns past the field or in a row's padding hold zeros, which stay zeros or are not
+      // stored; z tiles of odd rows have pairs across two rows
       const int plane = (int)((uint32_t)tile / (uint32_t)a.tiles_per_plane);
       const uint32_t cg = ((uint32_t)tile - (uint32_t)plane * (uint32_t)a.tiles_per_plane) *
-                              (uint32_t)CW + (uint32_t)c;
-      if (a.mode == 1) {
-        active = cg < (uint32_t)a.C;
-        s = (int)(cg % (uint32_t)S);
-        if (dir_after) {
-          const int x0 = (int)(cg / (uint32_t)S);
-          face = (x0 == 0 || x0 == a.nx - 1 || plane == 0 || plane == a.nz - 1);
+                              (uint32_t)CW + (uint32_t)col0;
+      if (!s_fixed || dir.any) {
+        uint32_t xs = cg, y = 0;
+        if (a.mode != 1) {
+          y = cg / (uint32_t)a.gpitch;
+          xs = cg - y * (uint32_t)a.gpitch;
         }
-      } else {  // a plane of ny rows gpitch apart: padding columns are not lines
-        const uint32_t y = cg / (uint32_t)a.gpitch, xs = cg - y * (uint32_t)a.gpitch;
-        active = cg < (uint32_t)a.C && xs < (uint32_t)a.rowlen;
-        s = (int)(xs % (uint32_t)S);
-        if (dir_after) {
-          const int x0 = (int)(xs / (uint32_t)S);
-          face = (x0 == 0 || x0 == a.nx - 1 || y == 0 || (int)y == a.ny - 1);
+        if (!s_fixed) set_substrates((int)(xs % (uint32_t)S), (int)((xs + 1) % (uint32_t)S));
+        if (dir.any) {
+          auto face = [&](uint32_t xs, uint32_t y) {
+            const bool edge = a.mode == 1 ? plane == 0 || plane == a.nz - 1
+                                          : y == 0 || (int)y == a.ny - 1;
+            const int x = (int)(xs / (uint32_t)S);
+            return x < a.nx && (edge || x == 0 || x == a.nx - 1);
+          };
+          dir.face0 = face(xs, y);
+          const bool next_row = a.mode != 1 && xs + 1 == (uint32_t)a.gpitch;
+          dir.face1 = next_row ? face(0, y + 1) : face(xs + 1, y);
         }
       }
     }
-    const int len = active ? len_full : 0;
-    H *p = stg + colbase + lo * ps_rt;
-    const int rowoff = s * npad + lo;
-    const bool dir = s_fixed ? dir_f : dir_after && a.dir_on[s];
-    const E dval = s_fixed ? dval_f : dir ? dir_value<E>(a.flags, a.dir_val, s) : E(0);
-    const E chi = s_fixed ? chi_f : __ldg(g_cfix + s), clo = s_fixed ? clo_f : __ldg(g_cfix + S + s);
-    // the unguarded path only when every lane of the warp has a full chunk:
-    // the choice is warp-uniform, so a warp never splits across the paths
-    constexpr int PS = MODE == 0 ? PSX : CW;
-    bool solved;
-    if (__all_sync(0xffffffffu, len == MAXM))
-      solved = pipe_chunk<E, MAXM, true, PS, CW>(p, ps_rt, len, lo, n, t, T, c, s_inv + rowoff,
-                                             s_mul + rowoff, s_pf + rowoff, s_pb + rowoff, Tcw, S,
-                                             s, chi, clo, s_end, s_beg, ncons, dir, face, dval, ok);
-    else
-      solved = pipe_chunk<E, MAXM, false, PS, CW>(p, ps_rt, len, lo, n, t, T, c, s_inv + rowoff,
-                                              s_mul + rowoff, s_pf + rowoff, s_pb + rowoff, Tcw, S,
-                                              s, chi, clo, s_end, s_beg, ncons, dir, face, dval, ok);
+    col.p0 = stg + off0;
+    col.p1 = stg + off1;
+    const bool solved =
+        fast ? pipe_chunk<MAXM, true, CPW, VEC>(col, len, lo, n, wc, W, q, p, cf, s_end, s_beg,
+                                                ncons, dir, st0, st1, ok)
+             : pipe_chunk<MAXM, false, CPW, VEC>(col, len, lo, n, wc, W, q, p, cf, s_end, s_beg,
+                                                 ncons, dir, st0, st1, ok);
     if (!solved) break;
     fence_proxy_async_smem();  // generic-proxy writes -> visible to the bulk store
-    mbar_arrive(&done[st]);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&done[st]);
   }
 }
 
-// x tiles with a compile-time substrate count: the default chunk length only
-// (each specialisation is a full copy of the kernel).
-template <int MAXM>
-constexpr bool pipe_x_specialised() {
-  return MAXM == 32;
-}
-// Tiles of 16 columns (long lines): the chunk capacities the planner offers them.
-template <int MAXM>
-constexpr bool pipe_half_tiles() {
-  return MAXM == 32 || MAXM == 64;
-}
-
-template <typename E, int MAXM, typename H = E>
-cudaError_t allow_pipe_smem(size_t bytes) {
-  cudaError_t e = cudaSuccess;
-  auto set = [&](const void *f) {
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  };
-  set((const void *)sweep_pipe_kernel<E, MAXM, 0, 0, 32, H>);
-  set((const void *)sweep_pipe_kernel<E, MAXM, 1, 0, 32, H>);
-  if constexpr (pipe_half_tiles<MAXM>()) {
-    set((const void *)sweep_pipe_kernel<E, MAXM, 0, 0, 16, H>);
-    set((const void *)sweep_pipe_kernel<E, MAXM, 1, 0, 16, H>);
-  }
-  if constexpr (pipe_x_specialised<MAXM>()) {
-    set((const void *)sweep_pipe_kernel<E, MAXM, 0, 1, 32, H>);
-    set((const void *)sweep_pipe_kernel<E, MAXM, 0, 2, 32, H>);
-    set((const void *)sweep_pipe_kernel<E, MAXM, 0, 4, 32, H>);
-    set((const void *)sweep_pipe_kernel<E, MAXM, 0, 8, 32, H>);
-  }
-  if constexpr (std::is_same<H, E>::value && pipe_half_tiles<MAXM>()) {
-    set((const void *)sweep_pipe_kernel<E, MAXM, 0, 1, 16>);
-    set((const void *)sweep_pipe_kernel<E, MAXM, 0, 2, 16>);
-    set((const void *)sweep_pipe_kernel<E, MAXM, 0, 4, 16>);
-    set((const void *)sweep_pipe_kernel<E, MAXM, 0, 8, 16>);
-  }
+// Chunk capacities: 8, 16 and 24 positions of 32-column tiles, 16 and 24
+// of 16-column ones.  x tiles know the substrate count at compile time where it
+// is 1, 2, 4 or 8 (their chunk starts must then be multiples of the positions
+// one access reads: the capacity, or 0).
+template <int MAXM, int CW, typename H, typename F>
+cudaError_t pipe_kernels(F &&f) {  // f(x kernel for S, S), ..., f(y/z kernel, -1)
+  cudaError_t e = f((const void *)sweep_pipe_kernel<MAXM, 0, 0, CW, H>, 0);
+  if (e == cudaSuccess) e = f((const void *)sweep_pipe_kernel<MAXM, 0, 1, CW, H>, 1);
+  if (e == cudaSuccess) e = f((const void *)sweep_pipe_kernel<MAXM, 0, 2, CW, H>, 2);
+  if (e == cudaSuccess) e = f((const void *)sweep_pipe_kernel<MAXM, 0, 4, CW, H>, 4);
+  if (e == cudaSuccess) e = f((const void *)sweep_pipe_kernel<MAXM, 0, 8, CW, H>, 8);
+  if (e == cudaSuccess) e = f((const void *)sweep_pipe_kernel<MAXM, 1, 0, CW, H>, -1);
   return e;
 }
 
-template <typename E, int MAXM, typename H = E>
+template <int MAXM, typename H>
+cudaError_t allow_pipe_smem(size_t bytes) {
+  auto set = [&](const void *k, int) {
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  };
+  cudaError_t e = pipe_kernels<MAXM, 32, H>(set);
+  if constexpr (MAXM >= 16)
+    if (e == cudaSuccess) e = pipe_kernels<MAXM, 16, H>(set);
+  return e;
+}
+
+template <int MAXM, int CW, typename H>
+cudaError_t launch_pipe_cw(const CUtensorMap &map, const PipeArgs &a, int grid, size_t smem,
+                           cudaStream_t st) {
+  constexpr int CPW = 64 / CW;
+  const int threads = ((a.tab.T + CPW - 1) / CPW + 1 + a.prep_warp) * 32;
+  if (threads > 32 * pipe_sm_warps(MAXM)) return cudaErrorInvalidConfiguration;
+  const int psx = (a.S == 1 || a.S == 2 || a.S == 4 || a.S == 8) ? a.S : 0;
+  void *args[] = {const_cast<CUtensorMap *>(&map), const_cast<PipeArgs *>(&a)};
+  const void *k = nullptr;
+  pipe_kernels<MAXM, CW, H>([&](const void *f, int s) {
+    if (s == (a.mode != 0 ? -1 : psx)) k = f;
+    return cudaSuccess;
+  });
+  return cudaLaunchKernel(k, dim3(grid), dim3(threads), args, smem, st);
+}
+
+template <int MAXM, typename H>
 cudaError_t launch_pipe_one(const CUtensorMap &map, const PipeArgs &a, int grid, size_t smem,
                             cudaStream_t st) {
-  const int cpw = a.cw == 16 ? 2 : 1;
-  const int threads = ((a.tab.T + cpw - 1) / cpw + 1 + a.prep_warp) * 32;
-  if (threads > PipeBound<E, MAXM>::threads) return cudaErrorInvalidConfiguration;
-  if (a.cw == 16) {
-    if constexpr (pipe_half_tiles<MAXM>()) {
-      if (a.mode != 0) {
-        sweep_pipe_kernel<E, MAXM, 1, 0, 16, H><<<grid, threads, smem, st>>>(map, a);
-        return cudaGetLastError();
-      }
-      if constexpr (std::is_same<H, E>::value) {  // x tiles: S at compile time where it can be
-        switch (a.S) {
-          case 1: sweep_pipe_kernel<E, MAXM, 0, 1, 16><<<grid, threads, smem, st>>>(map, a); return cudaGetLastError();
-          case 2: sweep_pipe_kernel<E, MAXM, 0, 2, 16><<<grid, threads, smem, st>>>(map, a); return cudaGetLastError();
-          case 4: sweep_pipe_kernel<E, MAXM, 0, 4, 16><<<grid, threads, smem, st>>>(map, a); return cudaGetLastError();
-          case 8: sweep_pipe_kernel<E, MAXM, 0, 8, 16><<<grid, threads, smem, st>>>(map, a); return cudaGetLastError();
-          default: break;
-        }
-      }
-      sweep_pipe_kernel<E, MAXM, 0, 0, 16, H><<<grid, threads, smem, st>>>(map, a);
-      return cudaGetLastError();
-    }
-    return cudaErrorInvalidConfiguration;
-  }
-  if (a.cw != 32) return cudaErrorInvalidConfiguration;
-  if (a.mode != 0) {
-    sweep_pipe_kernel<E, MAXM, 1, 0, 32, H><<<grid, threads, smem, st>>>(map, a);
-    return cudaGetLastError();
-  }
-  if constexpr (pipe_x_specialised<MAXM>()) {
-    switch (a.S) {
-      case 1: sweep_pipe_kernel<E, MAXM, 0, 1, 32, H><<<grid, threads, smem, st>>>(map, a); return cudaGetLastError();
-      case 2: sweep_pipe_kernel<E, MAXM, 0, 2, 32, H><<<grid, threads, smem, st>>>(map, a); return cudaGetLastError();
-      case 4: sweep_pipe_kernel<E, MAXM, 0, 4, 32, H><<<grid, threads, smem, st>>>(map, a); return cudaGetLastError();
-      case 8: sweep_pipe_kernel<E, MAXM, 0, 8, 32, H><<<grid, threads, smem, st>>>(map, a); return cudaGetLastError();
-      default: break;
-    }
-  }
-  sweep_pipe_kernel<E, MAXM, 0, 0, 32, H><<<grid, threads, smem, st>>>(map, a);
-  return cudaGetLastError();
+  if (a.cw == 32) return launch_pipe_cw<MAXM, 32, H>(map, a, grid, smem, st);
+  if constexpr (MAXM >= 16)
+    if (a.cw == 16) return launch_pipe_cw<MAXM, 16, H>(map, a, grid, smem, st);
+  return cudaErrorInvalidConfiguration;
 }
 
 }  // namespace bfv

@@ -27,6 +27,38 @@ namespace bfv {
 //     j*cw + c.
 //
 // Tile k of a CTA is tile blockIdx.x + k*gridDim.x of ntiles.
+//
+// The consumers work on pairs of columns (packed FP32 pairs), so the constants
+// come as pairs too: one class per pair of substrates that occurs -- S even:
+// (2c, 2c+1), S odd: (c, c+1 mod S), S = 1: (0, 0).  AxisTab::tabT holds, in
+// pairs (pipe_tab_pairs of them):
+//   constants   [classes][4]              interior inv' and mul; c_hi, c_lo
+//   inv', mul   [2][classes][npad]        of every position of every chunk (0 past the line)
+//   weights     [classes][W * chunks per warp][kWtN]  products of mul over whole chunks of
+//               the chunk's warp (1 for chunks past the line):
+//               kWtF0 this chunk; kWtF1 it and the one before; kWtFx all before it;
+//               kWtB1 it and the one after; kWtBx all after it
+//   pw          [classes][W]              all of a warp's chunks
+enum { kWtF0, kWtF1, kWtFx, kWtB1, kWtBx, kWtN };
+#if defined(__CUDACC__)
+#define BFV_HD __host__ __device__
+#else
+#define BFV_HD
+#endif
+BFV_HD constexpr int pipe_classes(int S) { return S > 1 && S % 2 == 0 ? S / 2 : S; }
+// (two pairs past a multiple of 16: neighbouring classes start in other banks, 16-byte aligned)
+BFV_HD constexpr int pipe_npad(int n) { return (n + 15) / 16 * 16 + 2; }
+// maxm: positions of a chunk.
+BFV_HD constexpr int pipe_tab_pairs(int maxm, int S, int W, int chunks_per_warp) {
+  return pipe_classes(S) * (4 + 2 * pipe_npad(W * chunks_per_warp * maxm) +
+                            W * chunks_per_warp * kWtN + W);
+}
+// Registers of a thread of chunk capacity maxm (the chunk pair takes 2 maxm): 80, 96 and 128 hold
+// the solve with few or no spills, and the warps an SM then has room for (its four register files
+// take whole warps) -- also the largest CTA.
+BFV_HD constexpr int pipe_regs(int maxm) { return maxm <= 8 ? 80 : maxm <= 16 ? 96 : 128; }
+BFV_HD constexpr int pipe_sm_warps(int maxm) { return 4 * (16384 / (pipe_regs(maxm) * 32)); }
+
 struct PipeArgs {
   int mode, n, S, nx, ny, nz;
   int cw;  // columns per tile: 32 or 16
@@ -43,6 +75,7 @@ struct PipeArgs {
   int stages;
   int64_t stage_elems;
   AxisTab tab;
+  int k0;  // positions k0 .. n-2 have the interior coefficients
   int flags;
   // mode 0: sources (CSR over rows) and the Dirichlet application before the solve
   const int64_t *src_row_off, *src_elem;

@@ -1,7 +1,5 @@
 // Instantiations of the persistent TMA-pipelined sweep (pipe.cuh) for fields
-// stored in 16 bits -- bf16 or fp16 -- with FP32 arithmetic and FP32 constants:
-// chunk capacities 32 and 64 (the planner rounds the chunk capacity of a 16-bit
-// handle up to 32, and takes 16-line tiles rather than chunks above 64).
+// stored in 16 bits -- bf16 or fp16 -- with FP32 arithmetic and FP32 constants.
 #include "pipe.cuh"
 
 namespace bfv {
@@ -9,8 +7,9 @@ namespace bfv {
 template <typename H>
 cudaError_t allow_pipe_smem_h16(int maxm, size_t bytes) {
   switch (maxm) {
-    case 32: return allow_pipe_smem<float, 32, H>(bytes);
-    case 64: return allow_pipe_smem<float, 64, H>(bytes);
+    case 8: return allow_pipe_smem<8, H>(bytes);
+    case 16: return allow_pipe_smem<16, H>(bytes);
+    case 24: return allow_pipe_smem<24, H>(bytes);
   }
   return cudaErrorInvalidValue;
 }
@@ -19,8 +18,9 @@ template <typename H>
 cudaError_t launch_pipe_h16(const CUtensorMap &map, const PipeArgs &a, int maxm, int grid,
                             size_t smem, cudaStream_t st) {
   switch (maxm) {
-    case 32: return launch_pipe_one<float, 32, H>(map, a, grid, smem, st);
-    case 64: return launch_pipe_one<float, 64, H>(map, a, grid, smem, st);
+    case 8: return launch_pipe_one<8, H>(map, a, grid, smem, st);
+    case 16: return launch_pipe_one<16, H>(map, a, grid, smem, st);
+    case 24: return launch_pipe_one<24, H>(map, a, grid, smem, st);
   }
   return cudaErrorInvalidValue;
 }
