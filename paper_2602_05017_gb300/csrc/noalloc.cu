@@ -115,13 +115,13 @@ extern "C" biofvm_status biofvm_param_grad_noalloc(const void *mu, const void *u
     bfv::adj_reduce_kernel<double><<<kBlocks, bfv::kReduceThreads, 0, st>>>(
         static_cast<const double *>(mu), static_cast<const double *>(u), nel, n_sub, stride,
         n_axis, used, partial);
-    bfv::adj_reduce_final_kernel<double><<<1, 32, 0, st>>>(partial, kBlocks, n_sub, -dt / 3.0,
+    bfv::adj_reduce_final_kernel<double><<<1, bfv::kReduceFinalThreads, 0, st>>>(partial, kBlocks, n_sub, -dt / 3.0,
                                                            -dt / (h_axis * h_axis), dlambda, dD);
   } else {
     bfv::adj_reduce_kernel<float><<<kBlocks, bfv::kReduceThreads, 0, st>>>(
         static_cast<const float *>(mu), static_cast<const float *>(u), nel, n_sub, stride, n_axis,
         used, partial);
-    bfv::adj_reduce_final_kernel<float><<<1, 32, 0, st>>>(partial, kBlocks, n_sub, -dt / 3.0,
+    bfv::adj_reduce_final_kernel<float><<<1, bfv::kReduceFinalThreads, 0, st>>>(partial, kBlocks, n_sub, -dt / 3.0,
                                                           -dt / (h_axis * h_axis), dlambda, dD);
   }
   const cudaError_t e = cudaGetLastError();

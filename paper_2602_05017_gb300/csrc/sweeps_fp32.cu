@@ -59,7 +59,7 @@ cudaError_t launch_adj_reduce_f32(const ReduceLaunch &a, cudaStream_t st) {
   adj_reduce_kernel<float><<<a.nblocks, kReduceThreads, 0, st>>>(
       static_cast<const float *>(a.mu), static_cast<const float *>(a.u), a.nel, a.S, a.stride,
       a.n_axis, a.used, a.partial);
-  adj_reduce_final_kernel<float><<<1, 32, 0, st>>>(a.partial, a.nblocks, a.S, a.scale_lambda, a.scale_D,
+  adj_reduce_final_kernel<float><<<1, kReduceFinalThreads, 0, st>>>(a.partial, a.nblocks, a.S, a.scale_lambda, a.scale_D,
                                             a.dlambda, a.dD);
   return cudaGetLastError();
 }

@@ -52,7 +52,7 @@ cudaError_t launch_adj_reduce_f64(const ReduceLaunch &a, cudaStream_t st) {
   adj_reduce_kernel<double><<<a.nblocks, kReduceThreads, 0, st>>>(
       static_cast<const double *>(a.mu), static_cast<const double *>(a.u), a.nel, a.S, a.stride,
       a.n_axis, a.used, a.partial);
-  adj_reduce_final_kernel<double><<<1, 32, 0, st>>>(a.partial, a.nblocks, a.S, a.scale_lambda, a.scale_D,
+  adj_reduce_final_kernel<double><<<1, kReduceFinalThreads, 0, st>>>(a.partial, a.nblocks, a.S, a.scale_lambda, a.scale_D,
                                             a.dlambda, a.dD);
   return cudaGetLastError();
 }
