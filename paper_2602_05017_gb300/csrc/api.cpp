@@ -143,11 +143,12 @@ struct biofvm {
   int stream_r8_mode = -1;
   int stream32_enabled = 0;  // FP32 streaming sweeps instead of the pipelined ones
   // small FP64 grids: whole biofvm_step calls in one cooperative launch (small.cu)
-  int small_enabled = 1, small_use = 0, small_grid = 0;
+  int small_enabled = 1, small_use = 0, small_grid = 0, small_warps = 1, small_maxm = 8, small_cluster = 0;
+  int small_planes = 0;  // small_planes.cu, with small_smem bytes of shared memory
   size_t small_smem = 0;
   DevBuf small_bar;
   int small_T[3] = {1, 1, 1}, small_m[3] = {1, 1, 1};  // chunks per axis of the small step
-  DevBuf small_tab[3];                                   // their axis tables
+  DevBuf small_tab[3];                                   // their tables (LineTab; small_planes: axis_tables)
   int pipe_chunk = 0;        // FP32 pipelined sweeps: chunk length (0: the planner's)
   int pipe_cw = 0;           // FP32 pipelined sweeps: lines per tile, 32 or 16 (0: the planner's)
   int pipe_ns = 4;           // FP32 pipelined sweeps: most ring stages per CTA
@@ -272,6 +273,51 @@ void axis_tables(const biofvm *h, int axis, int T, int m, bool defect, std::vect
         cw[((size_t)u * T + t) * S + s] = w;
       }
   }
+}
+
+// Tables of the warp-level line solves (LineTab) of one axis, T chunks of m positions:
+// inv, mul [T*m][S], scan weights [log2 T][2][T][S], c_hi, c_lo [2][S].
+void line_tables(const biofvm *h, int axis, int T, int m, bool defect, std::vector<double> &out) {
+  const int n = axis_len(h, axis), S = h->g.n_sub, np = T * m;
+  std::vector<double> t;
+  axis_tables(h, axis, (n + m - 1) / m, m, defect, t);
+  const int Tn = (n + m - 1) / m;  // chunks that hold positions
+  const double *inv = t.data(), *mul = inv + (size_t)n * S, *pc = mul + 3 * (size_t)n * S,
+               *cfix = pc + (size_t)Tn * S;
+  int lg = 0;
+  while ((1 << lg) < T) lg++;
+  out.assign((size_t)2 * np * S + (size_t)2 * lg * T * S + 2 * (size_t)S, 0.0);
+  double *wt = out.data() + (size_t)2 * np * S, *cf = wt + (size_t)2 * lg * T * S;
+  std::copy(inv, inv + (size_t)n * S, out.begin());
+  std::copy(mul, mul + (size_t)n * S, out.begin() + (size_t)np * S);
+  std::copy(cfix, cfix + 2 * (size_t)S, cf);
+  auto prod = [&](int lo, int hi, int s) {  // over whole chunks lo..hi
+    double x = 1.0;
+    for (int u = std::max(lo, 0); u <= hi; u++) x *= u < Tn ? pc[(size_t)u * S + s] : 0.0;
+    return x;
+  };
+  for (int k = 0; k < lg; k++)
+    for (int c = 0; c < T; c++)
+      for (int s = 0; s < S; s++) {
+        wt[((size_t)(2 * k) * T + c) * S + s] = prod(c - (1 << k) + 1, c, s);
+        wt[((size_t)(2 * k + 1) * T + c) * S + s] = prod(c, std::min(T - 1, c + (1 << k) - 1), s);
+      }
+}
+
+LineTab line_tab(const biofvm *h, int axis, int T, int m, const DevBuf &b) {
+  const int S = h->g.n_sub, np = T * m;
+  int lg = 0;
+  while ((1 << lg) < T) lg++;
+  const char *base = static_cast<const char *>(b.p);
+  LineTab t;
+  t.inv = base;
+  t.mul = base + (size_t)np * S * h->csz;
+  t.wt = base + (size_t)2 * np * S * h->csz;
+  t.cfix = base + ((size_t)2 * np * S + (size_t)2 * lg * T * S) * h->csz;
+  t.n = axis_len(h, axis);
+  t.T = T;
+  t.m = m;
+  return t;
 }
 
 // ---------------------------------------------------------------------------
@@ -605,26 +651,52 @@ void plan_stream(biofvm *h, int axis) {
   p.use = 1;
 }
 
-// Small FP64 grids (a field of at most 32 MB whose z-planes fit in shared
-// memory): biofvm_step runs all its steps in one cooperative launch.  The grid covers the z-planes and at least one CTA
-// per SM, within what can be co-resident.
+// Small FP64 grids: biofvm_step runs all its steps in one cooperative launch.
+// Lines of at most 128 voxels, a field of at most 12 MB (100^3: 63 us a step, 85 in streaming
+// sweeps; 128^3, 16.8 MB: 104 and 93): the warp-level solves of small.cu, one CTA per SM.
+// Longer lines, a field of at most 32 MB whose z-planes fit in shared memory: small_planes.cu,
+// the grid covering the z-planes and at least one CTA per SM.
 void plan_small(biofvm *h) {
-  h->small_use = 0;
+  h->small_use = h->small_planes = 0;
   if (!h->small_enabled || h->prec != BIOFVM_FP64 || h->forced) return;
   const int nx = h->g.nx, ny = h->g.ny, nz = h->g.nz, S = h->g.n_sub;
   if ((double)h->nel * 8.0 > 32.0e6 || !h->sp[2].use) return;
+  const int longest = std::max(nx, std::max(ny, nz));
+  if (longest <= 128) {
+    if ((double)h->nel * 8.0 > 12.0e6) return;
+    h->small_maxm = longest <= 64 ? 8 : 16;  // shorter chains and more warps for short lines
+    int64_t items = 1;
+    for (int a = 0; a < 3; a++) {
+      const int n = axis_len(h, a), T = line_chunks(n, h->small_maxm);
+      h->small_T[a] = T;
+      h->small_m[a] = (n + T - 1) / T;
+      items = std::max(items, ((int64_t)h->nel / n * T + 31) / 32);
+    }
+    if (dev_alloc(h->small_bar, 8) != cudaSuccess) {
+      cudaGetLastError();
+      return;
+    }
+    // few items: one cluster, whose barrier is the hardware's (20^3: 15.6 us a step, 17.3 on more
+    // SMs through the barrier in memory)
+    h->small_cluster = items <= 64;
+    h->small_grid = (int)std::min<int64_t>(h->small_cluster ? 8 : h->num_sms, items);
+    h->small_warps = (int)std::min<int64_t>(small_warps(h->small_maxm),
+                                            (items + h->small_grid - 1) / h->small_grid);
+    h->small_use = 1;
+    return;
+  }
   // chunks: x-lines ny*S per plane, y-lines nx*S, z-lines in groups of 32
   const int n3[3] = {nx, ny, nz}, L3[3] = {ny * S, nx * S, 32};
   int T[3];
   for (int a = 0; a < 3; a++) {
-    T[a] = small_chunks(n3[a], L3[a]);
+    T[a] = planes_chunks(n3[a], L3[a]);
     h->small_T[a] = T[a];
     h->small_m[a] = (n3[a] + T[a] - 1) / T[a];
   }
-  const size_t smem = small_smem_bytes(nx, ny, nz, S, T);
+  const size_t smem = planes_smem_bytes(nx, ny, nz, S, T);
   if (smem > 200 * 1024) return;
   int per_sm = 0;
-  if (small_max_blocks(&per_sm, smem) != cudaSuccess || per_sm < 1) {
+  if (planes_max_blocks(&per_sm, smem) != cudaSuccess || per_sm < 1) {
     cudaGetLastError();
     return;
   }
@@ -637,7 +709,7 @@ void plan_small(biofvm *h) {
   // barrier's cost grows with its CTAs
   const int groups = (int)(((int64_t)nx * ny * S + 31) / 32);
   h->small_grid = std::max(1, std::min(h->num_sms * per_sm, std::max(nz, groups)));
-  h->small_use = 1;
+  h->small_use = h->small_planes = 1;
 }
 
 // FP32 fields whose rows are not 16-byte multiples (the TMA copies' unit): a
@@ -836,9 +908,10 @@ biofvm_status upload_constants(biofvm *h) {
       return upload_doubles(h, dst, tt);
     };
     if ((st = upload_T(h->tabT[axis], h->pp[axis])) != BIOFVM_OK) return st;
-    if (h->small_use) {  // the small step's own chunk partition
+    if (h->small_use) {
       std::vector<double> ts;
-      axis_tables(h, axis, h->small_T[axis], h->small_m[axis], false, ts);
+      if (h->small_planes) axis_tables(h, axis, h->small_T[axis], h->small_m[axis], false, ts);
+      else line_tables(h, axis, h->small_T[axis], h->small_m[axis], f32, ts);
       if ((st = upload_doubles(h, h->small_tab[axis], ts)) != BIOFVM_OK) return st;
     }
     // the row-padded working copy's plans: tables of their own partition
@@ -1896,31 +1969,44 @@ biofvm_status biofvm_step(biofvm_t *h, int n_steps) {
   if (n_steps == 0) return BIOFVM_OK;
   CK(cudaSetDevice(h->device));
   if (h->small_use && h->n_dnode == 0) {  // one cooperative launch for all the steps
-    SmallArgs a{};
-    a.rho = static_cast<double *>(h->rho.p);
-    a.nx = h->g.nx;
-    a.ny = h->g.ny;
-    a.nz = h->g.nz;
-    a.S = h->g.n_sub;
-    for (int axis = 0; axis < 3; axis++) {
-      a.tab[axis] = static_cast<const double *>(h->small_tab[axis].p);
-      a.T[axis] = h->small_T[axis];
-      a.m[axis] = h->small_m[axis];
+    auto common = [&](auto &a) {
+      a.rho = static_cast<double *>(h->rho.p);
+      a.nx = h->g.nx;
+      a.ny = h->g.ny;
+      a.nz = h->g.nz;
+      a.S = h->g.n_sub;
+      const SrcLists sl = src_lists(h);
+      a.src_row_off = sl.row_off;
+      a.src_elem = sl.elem;
+      a.src_alpha = static_cast<const double *>(sl.alpha);
+      a.src_scale = static_cast<const double *>(sl.scale);
+      a.has_src = sl.has;
+      a.dir_on = static_cast<const uint8_t *>(h->dir_on_d.p);
+      a.dir_val = static_cast<const double *>(h->dir_val_d.p);
+      a.any_dir = h->any_dir ? 1 : 0;
+      a.n_steps = n_steps;
+      a.bar = static_cast<unsigned *>(h->small_bar.p);
+      a.status = static_cast<int *>(h->status.p);
+    };
+    if (h->small_planes) {
+      PlanesArgs a{};
+      common(a);
+      for (int axis = 0; axis < 3; axis++) {
+        a.tab[axis] = static_cast<const double *>(h->small_tab[axis].p);
+        a.T[axis] = h->small_T[axis];
+        a.m[axis] = h->small_m[axis];
+      }
+      CK(cudaMemsetAsync(h->small_bar.p, 0, 16, h->stream));
+      CK(launch_planes_f64(a, h->small_grid, h->small_smem, h->stream));
+      return BIOFVM_OK;
     }
-    const SrcLists sl = src_lists(h);
-    a.src_row_off = sl.row_off;
-    a.src_elem = sl.elem;
-    a.src_alpha = static_cast<const double *>(sl.alpha);
-    a.src_scale = static_cast<const double *>(sl.scale);
-    a.has_src = sl.has;
-    a.dir_on = static_cast<const uint8_t *>(h->dir_on_d.p);
-    a.dir_val = static_cast<const double *>(h->dir_val_d.p);
-    a.any_dir = h->any_dir ? 1 : 0;
-    a.n_steps = n_steps;
-    a.bar = static_cast<unsigned *>(h->small_bar.p);
-    a.status = static_cast<int *>(h->status.p);
-    CK(cudaMemsetAsync(h->small_bar.p, 0, 16, h->stream));
-    CK(launch_small_f64(a, h->small_grid, h->small_smem, h->stream));
+    SmallArgs a{};
+    common(a);
+    for (int axis = 0; axis < 3; axis++)
+      a.tab[axis] = line_tab(h, axis, h->small_T[axis], h->small_m[axis], h->small_tab[axis]);
+    if (!h->small_cluster) CK(cudaMemsetAsync(h->small_bar.p, 0, 8, h->stream));
+    CK(launch_small_f64(a, h->small_maxm, h->small_grid, 32 * h->small_warps,
+                        h->small_cluster != 0, h->stream));
     return BIOFVM_OK;
   }
   // graphs of K steps (a renormalisation block) and of a shorter tail, each

@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lines_args.h"
+
 namespace bfv {
 
 // Stage flags of the sweep kernels (the x-sweep also owns Src and the first
@@ -187,10 +189,31 @@ cudaError_t allow_stream_smem_f64();
 cudaError_t launch_stream_f64(const StreamArgs &a, int grid, cudaStream_t st);
 cudaError_t launch_stream_f32(const StreamArgs &a, int grid, cudaStream_t st);
 // Small FP64 grids: all steps of a call in one cooperative launch (small.cu).
+// bar: 2 words (arrivals, abort) of the bounded grid barrier, zeroed before each launch.
+struct SmallArgs {
+  double *rho;
+  int nx, ny, nz, S;
+  LineTab tab[3];
+  const int64_t *src_row_off, *src_elem;
+  const double *src_alpha, *src_scale;
+  int has_src;
+  const uint8_t *dir_on;
+  const double *dir_val;
+  int any_dir;
+  int n_steps;
+  unsigned *bar;
+  int *status;
+};
+// Warps of a CTA at most: 128 and 168 registers a thread for chunks of 8 and 16.
+constexpr int small_warps(int maxm) { return maxm <= 8 ? 16 : 12; }
+// cluster: one cluster of grid <= 8 CTAs, its own barrier; else a cooperative launch.
+cudaError_t launch_small_f64(const SmallArgs &a, int maxm, int grid, int threads, bool cluster,
+                             cudaStream_t st);
+// The same for grids with lines of more than 128 voxels (small_planes.cu).
 // Planes of nx*ny*S elements in shared memory for the x and y solves, z-lines
 // by the streaming line solver; bar: 3 words (arrivals, generation, abort) of
 // the bounded grid barrier, zeroed before each launch.
-struct SmallArgs {
+struct PlanesArgs {
   double *rho;
   int nx, ny, nz, S;
   // per axis: the host's chunked axis tables (inv, mul, pf, pb [n][S], pc [T][S],
@@ -207,10 +230,10 @@ struct SmallArgs {
   unsigned *bar;
   int *status;
 };
-int small_chunks(int n, int L);
-size_t small_smem_bytes(int nx, int ny, int nz, int S, const int T[3]);
-cudaError_t small_max_blocks(int *blocks_per_sm, size_t smem);
-cudaError_t launch_small_f64(const SmallArgs &a, int grid, size_t smem, cudaStream_t st);
+int planes_chunks(int n, int L);
+size_t planes_smem_bytes(int nx, int ny, int nz, int S, const int T[3]);
+cudaError_t planes_max_blocks(int *blocks_per_sm, size_t smem);
+cudaError_t launch_planes_f64(const PlanesArgs &a, int grid, size_t smem, cudaStream_t st);
 // Sets the thread-local message biofvm_last_error() returns.
 void set_error_message(const char *msg);
 
