@@ -76,7 +76,7 @@ struct ColPlan {
 // the plain kernels).
 struct PipePlan {
   int use = 0, T = 1, m = 1, maxm = 8;
-  int cw = 32, W = 1;  // columns per tile (32, or 16 for long lines); consumer warps
+  int cw = 32, W = 1;  // columns per tile (32, or 24 or 16 for long lines); consumer warps
   int box_rows = 0, nbox = 0, rows_per_tile = 0, pitch = 0;
   int stages = 0, ctas = 1, grid = 0;  // ctas: per SM
   int64_t stage_elems = 0, ntiles = 0;
@@ -509,18 +509,22 @@ void plan_pipe(biofvm *h, int axis, PipePlan &p, int64_t gp, void *field) {
   const size_t esz = h->esz;
   const int n = axis_len(h, axis);
   if (h->prec == BIOFVM_FP64) return;  // FP64 streams whole lines instead
-  for (int cw : {32, 16}) {
+  for (int cw : {32, 24, 16}) {
     if (h->pipe_cw && cw != h->pipe_cw) continue;
+    if (cw == 24 && axis == 0) continue;
     PipePlan q{};
     q.cw = cw;
-    const int cpw = 64 / cw;  // chunks per consumer warp
+    const int cpw = pipe_chunks_per_warp(cw);
     const int extra = axis == 0 ? 2 : 1;  // warps besides the consumers: producer (+ preparer)
-    // chunks of exactly the capacity (the last one shorter), 16 positions where their warps fit
-    // in a CTA, else 24 (positions past the line's end have zero coefficients)
+    // chunks of exactly the capacity (the last one shorter; positions past the line's end have
+    // zero coefficients), the shortest whose warps fit in a CTA.  48 positions (y/z) keep long
+    // lines on tiles of 32 or 24 columns: z sweeps read one tile row per plane, and with 16
+    // columns, 64 bytes, a 1200 x 400 x 900 x 2 sweep ran at 2.5 TB/s (with 24 at 3.7).
     bool found = false;
-    for (int target : {16, 24}) {
+    for (int target : {16, 24, 48}) {
       const int want = h->pipe_chunk > 0 ? h->pipe_chunk : target;
-      q.m = q.maxm = want <= 8 && cw == 32 ? 8 : want <= 16 ? 16 : 24;
+      q.m = q.maxm = want <= 8 && cw == 32 ? 8 : want <= 16 ? 16 : want <= 24 ? 24 : 48;
+      if (q.maxm == 48 ? axis == 0 || cw == 16 : cw == 24) continue;
       q.T = (n + q.m - 1) / q.m;
       q.W = (q.T + cpw - 1) / cpw;
       if (q.W + extra > pipe_sm_warps(q.maxm)) continue;
@@ -557,7 +561,7 @@ void plan_pipe(biofvm *h, int axis, PipePlan &p, int64_t gp, void *field) {
       // 128-byte aligned, so box_rows * cw * esz is rounded up to a 128-byte multiple (rows
       // past the line's end are filled with zeros on load and skipped on store)
       q.nbox = (n + 255) / 256;
-      const int rgran = std::max(1, (int)(128 / ((size_t)cw * esz)));
+      const int rgran = cw == 24 ? (int)(16 / esz) : std::max(1, (int)(128 / ((size_t)cw * esz)));
       q.box_rows = ((n + q.nbox - 1) / q.nbox + rgran - 1) / rgran * rgran;
       if (((size_t)q.box_rows * cw * esz) % 128 != 0 || q.box_rows > 256) continue;
       q.stage_elems = (int64_t)q.nbox * q.box_rows * cw;
@@ -566,8 +570,8 @@ void plan_pipe(biofvm *h, int axis, PipePlan &p, int64_t gp, void *field) {
     }
     const size_t stage = (size_t)q.stage_elems * esz;
     const size_t tab = (size_t)pipe_tab_pairs(q.maxm, (int)S, q.W, cpw) * 8 + 16;  // + alignment
-    // carry exchange [2][W][cw/2] pairs; mbarriers: full, done, ready per stage, at most 8 stages
-    const size_t scratch = 2 * (size_t)q.W * (cw / 2) * 8 + 3 * 8 * 8;
+    // carry exchange [2][W][32 / cpw] pairs; mbarriers: full, done, ready per stage, at most 8 stages
+    const size_t scratch = 2 * (size_t)q.W * (32 / cpw) * 8 + 3 * 8 * 8;
     // As many CTAs per SM as the registers take, while each keeps three stages (256 positions:
     // two CTAs of 9 warps); else one with as many stages as fit.
     const int most = std::max(2, std::min(h->pipe_ns, 8));
@@ -867,7 +871,7 @@ biofvm_status upload_constants(biofvm *h) {
     auto upload_T = [&](DevBuf &dst, const PipePlan &q) -> biofvm_status {
       if (!q.use) return BIOFVM_OK;
       const int n = axis_len(h, axis), S = h->g.n_sub;
-      const int ncls = pipe_classes(S), cpw = 64 / q.cw, nch = q.W * cpw;
+      const int ncls = pipe_classes(S), cpw = pipe_chunks_per_warp(q.cw), nch = q.W * cpw;
       const int npad = pipe_npad(nch * q.maxm);
       std::vector<double> tt((size_t)2 * pipe_tab_pairs(q.maxm, S, q.W, cpw), 0.0);
       const double *inv = t.data(), *mul = inv + (size_t)n * S;

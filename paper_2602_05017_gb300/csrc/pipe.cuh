@@ -3,8 +3,8 @@
 // The arithmetic is the plain kernels' of sweeps.cuh -- partitioned Thomas of
 // Algorithm 1 on the App. A system, FP32 in defect-correction form -- on tiles
 // of CW independent lines ("columns") x n positions that move through a ring
-// of shared-memory stages.  CW = 32 normally; 16 for lines so long that two
-// stages of 32 columns do not fit:
+// of shared-memory stages.  CW = 32 normally; 24 (y/z) or 16 for lines so long
+// that two stages of 32 columns do not fit:
 //
 //   warp 0 (producer): TMA loads of tile k+NS-1 (cp.async.bulk.tensor boxes
 //     for y/z tiles, issued by lane 0; one cp.async.bulk per row for x tiles,
@@ -19,7 +19,8 @@
 //     instead of `full`;
 //   the next W warps (consumers): each thread holds one chunk (MAXM positions)
 //     of a PAIR of columns in registers and works on both with packed FP32
-//     instructions; a warp holds 64/CW chunks of the tile's CW/2 pairs.
+//     instructions; a warp holds two chunks (CW = 16: four) of the
+//     tile's CW/2 pairs.
 //     Carries cross a warp by shuffles and the CTA through shared memory,
 //     between two named barriers per tile that only consumers join.
 //
@@ -453,10 +454,10 @@ __device__ __forceinline__ bool pipe_chunk(const Cols col, const int len, const 
 template <int MAXM, int MODE, int PSX = 0, int CW = 32, typename H = float>
 __global__ void __maxnreg__(pipe_regs(MAXM))
     sweep_pipe_kernel(const __grid_constant__ CUtensorMap map, const PipeArgs a) {
-  static_assert(CW == 32 || CW == 16, "tiles of 32 or 16 columns");
+  static_assert(CW == 32 || CW == 24 || CW == 16, "tiles of 32, 24 or 16 columns");
   typedef float E;
-  constexpr int CPW = 64 / CW;    // chunks per consumer warp
-  constexpr int PW = 32 / CPW;    // column pairs of the tile
+  constexpr int CPW = pipe_chunks_per_warp(CW);
+  constexpr int PW = 32 / CPW;    // lanes of a chunk, one per column pair (CW = 24: four idle)
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int T = a.tab.T, n = a.n, S = a.S, NS = a.stages;
   const int64_t stage_elems = a.stage_elems;
@@ -831,19 +832,24 @@ __global__ void __maxnreg__(pipe_regs(MAXM))
 }
 
 // Chunk capacities: 8, 16 and 24 positions of 32-column tiles, 16 and 24
-// of 16-column ones.  x tiles know the substrate count at compile time where it
+// of 16-column ones; y/z tiles of 32 and 24 columns also 48 (lines whose
+// shorter chunks would take more warps than fit).  x tiles know the substrate count at compile time where it
 // is 1, 2, 4 or 8 (their chunk starts must then be multiples of the positions
 // one access reads: the capacity, or 0).
 template <int MAXM, int CW, typename H, typename F>
 cudaError_t pipe_kernels(F &&f) {  // f(x kernel for S, S), ..., f(y/z kernel, -1)
-  cudaError_t e = f((const void *)sweep_pipe_kernel<MAXM, 0, 0, CW, H>, 0);
-  if (e == cudaSuccess) e = f((const void *)sweep_pipe_kernel<MAXM, 0, 1, CW, H>, 1);
-  if (e == cudaSuccess) e = f((const void *)sweep_pipe_kernel<MAXM, 0, 2, CW, H>, 2);
-  if (e == cudaSuccess) e = f((const void *)sweep_pipe_kernel<MAXM, 0, 4, CW, H>, 4);
-  if (e == cudaSuccess) e = f((const void *)sweep_pipe_kernel<MAXM, 0, 8, CW, H>, 8);
-  if (e == cudaSuccess) e = f((const void *)sweep_pipe_kernel<MAXM, 1, 0, CW, H>, -1);
+  cudaError_t e = f((const void *)sweep_pipe_kernel<MAXM, 1, 0, CW, H>, -1);
+  if constexpr (MAXM <= 24) {
+    if (e == cudaSuccess) e = f((const void *)sweep_pipe_kernel<MAXM, 0, 0, CW, H>, 0);
+    if (e == cudaSuccess) e = f((const void *)sweep_pipe_kernel<MAXM, 0, 1, CW, H>, 1);
+    if (e == cudaSuccess) e = f((const void *)sweep_pipe_kernel<MAXM, 0, 2, CW, H>, 2);
+    if (e == cudaSuccess) e = f((const void *)sweep_pipe_kernel<MAXM, 0, 4, CW, H>, 4);
+    if (e == cudaSuccess) e = f((const void *)sweep_pipe_kernel<MAXM, 0, 8, CW, H>, 8);
+  }
   return e;
 }
+// The second tile width of a capacity (0: none).
+constexpr int pipe_narrow(int maxm) { return maxm <= 8 ? 0 : maxm <= 24 ? 16 : 24; }
 
 template <int MAXM, typename H>
 cudaError_t allow_pipe_smem(size_t bytes) {
@@ -851,15 +857,15 @@ cudaError_t allow_pipe_smem(size_t bytes) {
     return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   };
   cudaError_t e = pipe_kernels<MAXM, 32, H>(set);
-  if constexpr (MAXM >= 16)
-    if (e == cudaSuccess) e = pipe_kernels<MAXM, 16, H>(set);
+  if constexpr (pipe_narrow(MAXM) > 0)
+    if (e == cudaSuccess) e = pipe_kernels<MAXM, pipe_narrow(MAXM), H>(set);
   return e;
 }
 
 template <int MAXM, int CW, typename H>
 cudaError_t launch_pipe_cw(const CUtensorMap &map, const PipeArgs &a, int grid, size_t smem,
                            cudaStream_t st) {
-  constexpr int CPW = 64 / CW;
+  constexpr int CPW = pipe_chunks_per_warp(CW);
   const int threads = ((a.tab.T + CPW - 1) / CPW + 1 + a.prep_warp) * 32;
   if (threads > 32 * pipe_sm_warps(MAXM)) return cudaErrorInvalidConfiguration;
   const int psx = (a.S == 1 || a.S == 2 || a.S == 4 || a.S == 8) ? a.S : 0;
@@ -869,6 +875,7 @@ cudaError_t launch_pipe_cw(const CUtensorMap &map, const PipeArgs &a, int grid, 
     if (s == (a.mode != 0 ? -1 : psx)) k = f;
     return cudaSuccess;
   });
+  if (!k) return cudaErrorInvalidConfiguration;
   return cudaLaunchKernel(k, dim3(grid), dim3(threads), args, smem, st);
 }
 
@@ -876,8 +883,9 @@ template <int MAXM, typename H>
 cudaError_t launch_pipe_one(const CUtensorMap &map, const PipeArgs &a, int grid, size_t smem,
                             cudaStream_t st) {
   if (a.cw == 32) return launch_pipe_cw<MAXM, 32, H>(map, a, grid, smem, st);
-  if constexpr (MAXM >= 16)
-    if (a.cw == 16) return launch_pipe_cw<MAXM, 16, H>(map, a, grid, smem, st);
+  if constexpr (pipe_narrow(MAXM) > 0)
+    if (a.cw == pipe_narrow(MAXM))
+      return launch_pipe_cw<MAXM, pipe_narrow(MAXM), H>(map, a, grid, smem, st);
   return cudaErrorInvalidConfiguration;
 }
 

@@ -7,7 +7,7 @@
 namespace bfv {
 
 // A tile is cw "columns" (independent lines) x n positions along the axis,
-// cw = 32, or 16 for lines too long for two stages of 32 columns.
+// cw = 32, or 24 (y/z) or 16 for lines too long for two stages of 32 columns.
 //
 // The field's rows (fixed y, z: rowlen = nx*S elements) start gpitch elements
 // apart in global memory: gpitch = rowlen, or rowlen rounded up to 16 bytes for
@@ -45,6 +45,9 @@ enum { kWtF0, kWtF1, kWtFx, kWtB1, kWtBx, kWtN };
 #else
 #define BFV_HD
 #endif
+// Chunks of a tile that a consumer warp holds: its 12 or 16 column pairs side by side take half
+// a warp, 8 a quarter.
+BFV_HD constexpr int pipe_chunks_per_warp(int cw) { return cw == 16 ? 4 : 2; }
 BFV_HD constexpr int pipe_classes(int S) { return S > 1 && S % 2 == 0 ? S / 2 : S; }
 // (two pairs past a multiple of 16: neighbouring classes start in other banks, 16-byte aligned)
 BFV_HD constexpr int pipe_npad(int n) { return (n + 15) / 16 * 16 + 2; }
@@ -53,15 +56,15 @@ BFV_HD constexpr int pipe_tab_pairs(int maxm, int S, int W, int chunks_per_warp)
   return pipe_classes(S) * (4 + 2 * pipe_npad(W * chunks_per_warp * maxm) +
                             W * chunks_per_warp * kWtN + W);
 }
-// Registers of a thread of chunk capacity maxm (the chunk pair takes 2 maxm): 80, 96 and 128 hold
-// the solve with few or no spills, and the warps an SM then has room for (its four register files
+// Registers of a thread of chunk capacity maxm (the chunk pair takes 2 maxm): 80, 96, 128 and 168
+// hold the solve with few or no spills, and the warps an SM then has room for (its four register files
 // take whole warps) -- also the largest CTA.
-BFV_HD constexpr int pipe_regs(int maxm) { return maxm <= 8 ? 80 : maxm <= 16 ? 96 : 128; }
+BFV_HD constexpr int pipe_regs(int maxm) { return maxm <= 8 ? 80 : maxm <= 16 ? 96 : maxm <= 24 ? 128 : 168; }
 BFV_HD constexpr int pipe_sm_warps(int maxm) { return 4 * (16384 / (pipe_regs(maxm) * 32)); }
 
 struct PipeArgs {
   int mode, n, S, nx, ny, nz;
-  int cw;  // columns per tile: 32 or 16
+  int cw;  // columns per tile: 32, 24 or 16
   int64_t ntiles;
   // mode 1 / 2
   int64_t C;

@@ -10,6 +10,7 @@ cudaError_t allow_pipe_smem_h16(int maxm, size_t bytes) {
     case 8: return allow_pipe_smem<8, H>(bytes);
     case 16: return allow_pipe_smem<16, H>(bytes);
     case 24: return allow_pipe_smem<24, H>(bytes);
+    case 48: return allow_pipe_smem<48, H>(bytes);
   }
   return cudaErrorInvalidValue;
 }
@@ -21,6 +22,7 @@ cudaError_t launch_pipe_h16(const CUtensorMap &map, const PipeArgs &a, int maxm,
     case 8: return launch_pipe_one<8, H>(map, a, grid, smem, st);
     case 16: return launch_pipe_one<16, H>(map, a, grid, smem, st);
     case 24: return launch_pipe_one<24, H>(map, a, grid, smem, st);
+    case 48: return launch_pipe_one<48, H>(map, a, grid, smem, st);
   }
   return cudaErrorInvalidValue;
 }
