@@ -299,20 +299,26 @@ __device__ __forceinline__ f2 scan_bwd(f2 B, int q, const f2 *wt) {
 // time from the true carry costs one packed FMA per position -- the products
 // pf, pb that would correct the first result cost the same FMA and a
 // shared-memory load each.
-// FAST: MAXM positions of constant coefficients strictly inside the line.
+// KIND kInner: MAXM positions of constant coefficients strictly inside the line;
+// kFull: MAXM positions, coefficients from the tables; kRagged: any chunk.
 // Returns false when a consumer's wait for the tile timed out.
-template <int MAXM, bool FAST, int CPW, int VEC, typename Cols>
+enum { kInner, kFull, kRagged };
+template <int MAXM, int KIND, int CPW, int VEC, typename Cols>
 __device__ __forceinline__ bool pipe_chunk(const Cols col, const int len, const int lo,
                                            const int n, const int wc, const int W, const int q,
                                            const int p, const PairCoef &cf, f2 *s_end,
                                            f2 *s_beg, const int ncons, const PairDir &dir,
                                            const bool st0, const bool st1, const bool ok) {
   constexpr int PW = 32 / CPW;
+  constexpr bool FAST = KIND == kInner;
   const unsigned FULL = 0xffffffffu;
   f2 v[MAXM];
   const f2 zero = 0;
   f2 g = zero;
-  auto at = [&](int i) { return col.one(max(-lo, min(i, n - 1 - lo))); };  // position clamped
+  auto at = [&](int i) {  // position i, clamped to the line
+    if (KIND == kFull && i >= 0 && i < MAXM) return col.one(i);
+    return col.one(max(-lo, min(i, n - 1 - lo)));
+  };
   if constexpr (FAST) {
     const f2 c0 = cf.K[0], c1 = cf.K[1];
     const f2 before = col.one(-1), after = col.one(MAXM);
@@ -436,7 +442,7 @@ __device__ __forceinline__ bool pipe_chunk(const Cols col, const int len, const 
           f2 r = f2_fma(chi, d, f2_fma(clo, d, x));
           if constexpr (decltype(dirc)::value)
             r = with_dir(r, lo + k == 0 || lo + k == n - 1);
-          col.put(k, r, st0 && k < len, st1 && k < len);
+          col.put(k, r, st0 && (KIND == kFull || k < len), st1 && (KIND == kFull || k < len));
         }
       }
     };
@@ -709,8 +715,12 @@ __global__ void __maxnreg__(pipe_regs(MAXM))
   ColPair<H, PS, kPair, VEC> col;
   col.ps_rt = MODE == 0 ? S : CW;
   const int off0 = offset(col0) + lo * col.ps(), off1 = offset(col1) + lo * col.ps();
-  // constant coefficients strictly inside the line, for the whole warp
-  const bool fast = __all_sync(0xffffffffu, len == MAXM && lo >= max(a.k0, 1) && lo + MAXM <= n - 1);
+  // The kind of the warp's chunks.  Full chunks at a line's ends run unclamped only in 16-bit
+  // fields, which the solve bounds, not HBM (320 x 256 x 288 x 4, FP16: 94-119 us a sweep, 101-132
+  // clamped); in FP32 the third copy of the solve cost 1% at 400^3 x 4 and 5% over 48 ragged grids.
+  constexpr bool kHasFull = !std::is_same<H, float>::value;
+  const bool inner = __all_sync(0xffffffffu, len == MAXM && lo >= max(a.k0, 1) && lo + MAXM <= n - 1);
+  const bool full_chunks = kHasFull && __all_sync(0xffffffffu, len == MAXM);
   const bool dir_after = (a.flags & kDirAfter) != 0;
   const int ctid = threadIdx.x - 32 * cons0;  // consumer thread
   long long cn0 = 0, cn1 = 0;                 // entry range of the next tile (dense check)
@@ -819,11 +829,15 @@ __global__ void __maxnreg__(pipe_regs(MAXM))
     }
     col.p0 = stg + off0;
     col.p1 = stg + off1;
-    const bool solved =
-        fast ? pipe_chunk<MAXM, true, CPW, VEC>(col, len, lo, n, wc, W, q, p, cf, s_end, s_beg,
-                                                ncons, dir, st0, st1, ok)
-             : pipe_chunk<MAXM, false, CPW, VEC>(col, len, lo, n, wc, W, q, p, cf, s_end, s_beg,
-                                                 ncons, dir, st0, st1, ok);
+    bool solved;
+    if (kHasFull && full_chunks && !inner)
+      solved = pipe_chunk<MAXM, kHasFull ? kFull : kRagged, CPW, VEC>(
+          col, len, lo, n, wc, W, q, p, cf, s_end, s_beg, ncons, dir, st0, st1, ok);
+    else
+      solved = inner ? pipe_chunk<MAXM, kInner, CPW, VEC>(col, len, lo, n, wc, W, q, p, cf, s_end,
+                                                          s_beg, ncons, dir, st0, st1, ok)
+                     : pipe_chunk<MAXM, kRagged, CPW, VEC>(col, len, lo, n, wc, W, q, p, cf, s_end,
+                                                           s_beg, ncons, dir, st0, st1, ok);
     if (!solved) break;
     fence_proxy_async_smem();  // generic-proxy writes -> visible to the bulk store
     __syncwarp();
