@@ -59,7 +59,10 @@ struct DevBuf {
   }
 };
 
+// A buffer that is large enough, and less than twice too large, is kept: cudaFree waits for the
+// device, and a program that changes its agents or rates on every call would pay it each time.
 cudaError_t dev_alloc(DevBuf &b, size_t bytes) {
+  if (b.p && bytes > 0 && b.bytes >= bytes && b.bytes / 2 < bytes) return cudaSuccess;
   b.release();
   if (bytes == 0) return cudaSuccess;
   cudaError_t e = cudaMalloc(&b.p, bytes);
@@ -178,7 +181,8 @@ struct biofvm {
   DevBuf adj, partial, ag_elem, ag_entry, ag_weight, ag_target;
   int reduce_blocks = 0;
   bool agents_on_device = false;
-  std::vector<int64_t> h_voxel, h_src_elem;
+  std::vector<int64_t> h_voxel;
+  std::vector<int64_t> h_entry;  // per (agent, substrate): its element's source entry, or -1
   std::vector<double> h_weight, h_target;
   // the agents as last given (the source list is rebuilt when the nodes change)
   std::vector<double> h_secretion, h_uptake;
@@ -1316,48 +1320,66 @@ biofvm_status launch_step(const biofvm *h, cudaStream_t st, int m = 0, bool reno
 biofvm_status build_sources(biofvm *h) {
   const int S = h->g.n_sub;
   const int64_t n = (int64_t)h->h_voxel.size();
-  struct Ent {
-    int64_t e;
-    double alpha, beta;
-  };
-  std::vector<Ent> ent;
-  ent.reserve((size_t)n * S);
+  // each (agent, substrate)'s alpha and beta, rounded before they are summed
+  std::vector<double> pa((size_t)n * S), pb((size_t)n * S);
   for (int64_t k = 0; k < n; k++) {
     const double w = h->h_weight.empty() ? 1.0 : h->h_weight[k];
     for (int s = 0; s < S; s++) {
       const double sv = h->h_secretion[k * S + s], uv = h->h_uptake[k * S + s];
-      const double tv = h->h_target[k * S + s];
-      const double alpha = h->dt * w * sv * tv, beta = h->dt * w * (sv + uv);
-      const int64_t e = h->h_voxel[k] * S + s;
-      if ((alpha != 0.0 || beta != 0.0) &&
-          !std::binary_search(h->h_dn_kelem.begin(), h->h_dn_kelem.end(), e))
-        ent.push_back({e, alpha, beta});
+      pa[k * S + s] = h->dt * w * sv * h->h_target[k * S + s];
+      pb[k * S + s] = h->dt * w * (sv + uv);
     }
   }
-  std::stable_sort(ent.begin(), ent.end(), [](const Ent &a, const Ent &b) { return a.e < b.e; });
-  size_t u = 0;
-  for (size_t i = 0; i < ent.size(); i++) {
-    if (u > 0 && ent[u - 1].e == ent[i].e) {
-      ent[u - 1].alpha += ent[i].alpha;
-      ent[u - 1].beta += ent[i].beta;
-    } else {
-      ent[u++] = ent[i];
-    }
+  // The agents in voxel order, equal voxels in agent order, by a radix sort of 11 bits a pass: a
+  // voxel's agents are then neighbours, and its elements follow one another.  (A comparison sort
+  // of the S entries per agent and a search per entry for the adjoint's map took 1.1 ms more of
+  // a differentiable run with 40000 entries, 14 ms in all.)
+  std::vector<int64_t> order(n), tmp(n);
+  for (int64_t k = 0; k < n; k++) order[k] = k;
+  const int64_t nvox = (int64_t)h->g.nx * h->g.ny * h->g.nz;
+  for (int shift = 0; shift < 63 && ((nvox - 1) >> shift) > 0; shift += 11) {
+    int64_t at[2049] = {0};
+    auto digit = [&](int64_t k) { return (h->h_voxel[k] >> shift) & 2047; };
+    for (int64_t k = 0; k < n; k++) at[digit(k) + 1]++;
+    for (int d = 0; d < 2048; d++) at[d + 1] += at[d];
+    for (int64_t i = 0; i < n; i++) tmp[at[digit(order[i])]++] = order[i];
+    order.swap(tmp);
   }
-  ent.resize(u);
   const int64_t rowlen = (int64_t)h->g.nx * S;
   const int64_t nrows = (int64_t)h->g.ny * h->g.nz;
-  std::vector<int64_t> off(nrows + 1, 0), elem(u);
-  std::vector<int32_t> rowcol(2 * u);  // (row, position in the row) of each entry
-  std::vector<double> alpha(u), scale(u);
-  for (size_t i = 0; i < u; i++) {
-    off[ent[i].e / rowlen + 1]++;
-    elem[i] = ent[i].e;
-    rowcol[2 * i] = (int32_t)(ent[i].e / rowlen);
-    rowcol[2 * i + 1] = (int32_t)(ent[i].e % rowlen);
-    alpha[i] = ent[i].alpha;
-    scale[i] = 1.0 / (1.0 + ent[i].beta);
+  std::vector<int64_t> off(nrows + 1, 0), elem, entry((size_t)n * S, -1);
+  std::vector<int32_t> rowcol;  // (row, position in the row) of each entry
+  std::vector<double> alpha, scale;
+  elem.reserve((size_t)n * S);
+  alpha.reserve((size_t)n * S);
+  scale.reserve((size_t)n * S);
+  rowcol.reserve(2 * (size_t)n * S);
+  for (int64_t i0 = 0, i1; i0 < n; i0 = i1) {
+    const int64_t voxel = h->h_voxel[order[i0]];
+    for (i1 = i0 + 1; i1 < n && h->h_voxel[order[i1]] == voxel;) i1++;
+    for (int s = 0; s < S; s++) {
+      double al = 0.0, be = 0.0;
+      bool any = false;
+      for (int64_t i = i0; i < i1; i++) {  // in agent order
+        const double a = pa[order[i] * S + s], b = pb[order[i] * S + s];
+        if (a == 0.0 && b == 0.0) continue;
+        al = any ? al + a : a;
+        be = any ? be + b : b;
+        any = true;
+      }
+      const int64_t e = voxel * S + s;
+      if (!any || std::binary_search(h->h_dn_kelem.begin(), h->h_dn_kelem.end(), e)) continue;
+      for (int64_t i = i0; i < i1; i++) entry[order[i] * S + s] = (int64_t)elem.size();
+      const int64_t row = e / rowlen;
+      off[row + 1]++;
+      elem.push_back(e);
+      rowcol.push_back((int32_t)row);
+      rowcol.push_back((int32_t)(e - row * rowlen));
+      alpha.push_back(al);
+      scale.push_back(1.0 / (1.0 + be));
+    }
   }
+  const size_t u = elem.size();
   for (int64_t r = 0; r < nrows; r++) off[r + 1] += off[r];
   CK(cudaStreamSynchronize(h->stream));  // the kernels may still read the old lists
   h->n_entries = 0;
@@ -1377,7 +1399,7 @@ biofvm_status build_sources(biofvm *h) {
     if (st) return st;
   }
   h->n_entries = (int64_t)u;
-  h->h_src_elem = elem;
+  h->h_entry.swap(entry);
   h->sources_device = false;
   h->agents_on_device = false;  // the adjoint's agent-to-entry map follows the list
   h->generation++;
@@ -2160,14 +2182,11 @@ biofvm_status biofvm_adjoint_step_rates(biofvm_t *h, const void *grad_out, void 
   }
   const int64_t na = (int64_t)h->h_voxel.size();
   if (!h->agents_on_device && na > 0) {
-    std::vector<int64_t> el((size_t)na * S), en((size_t)na * S);
+    std::vector<int64_t> el((size_t)na * S);
+    const std::vector<int64_t> &en = h->h_entry;
     for (int64_t k = 0; k < na; k++)
-      for (int s = 0; s < S; s++) {
-        const int64_t e = h->h_voxel[k] * S + s;
-        auto it = std::lower_bound(h->h_src_elem.begin(), h->h_src_elem.end(), e);
-        el[k * S + s] = e;
-        en[k * S + s] = (it != h->h_src_elem.end() && *it == e) ? (it - h->h_src_elem.begin()) : -1;
-      }
+      for (int s = 0; s < S; s++) el[k * S + s] = h->h_voxel[k] * S + s;
+    CK(cudaStreamSynchronize(st));  // an earlier adjoint step may still read the old arrays
     if (dev_alloc(h->ag_elem, el.size() * 8) != cudaSuccess ||
         dev_alloc(h->ag_entry, en.size() * 8) != cudaSuccess ||
         dev_alloc(h->ag_target, h->h_target.size() * 8) != cudaSuccess ||
