@@ -1280,16 +1280,34 @@ cudaError_t launch_nodes(const biofvm *h, cudaStream_t st, int m, int row, bool 
 // x-sweep stands for the node part of the application between Src and X^-1
 // (the source list holds no node element, and the fused face application
 // skips every substrate with a node on its faces, so the order holds).
-// The field into its row-padded working copy (in) or back (out).
-cudaError_t pitch_copy(const biofvm *h, bool in, cudaStream_t st) {
+// A field-shaped array (the field itself when NULL) into the row-padded working copy (in) or
+// back (out).
+cudaError_t pitch_copy(const biofvm *h, bool in, cudaStream_t st, void *field = nullptr) {
   const int64_t rows = (int64_t)h->g.ny * h->g.nz;
   const int rowlen = h->g.nx * h->g.n_sub;
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((rows + 7) / 8, 8 * h->num_sms));
-  return in ? launch_pitch_rows(h->rho.p, h->prow.p, rows, rowlen, rowlen, h->gpitch, h->esz,
-                                grid, st)
-            : launch_pitch_rows(h->prow.p, h->rho.p, rows, rowlen, h->gpitch, rowlen, h->esz,
-                                grid, st);
+  if (!field) field = h->rho.p;
+  return in ? launch_pitch_rows(field, h->prow.p, rows, rowlen, rowlen, h->gpitch, h->esz, grid, st)
+            : launch_pitch_rows(h->prow.p, field, rows, rowlen, h->gpitch, rowlen, h->esz, grid, st);
 }
+
+// The source update alone, on the field (no Dirichlet application).
+cudaError_t launch_src(const biofvm *h, cudaStream_t st) {
+  const SrcLists sl = src_lists(h);
+  if (!sl.has) return cudaSuccess;
+  SrcLaunch a{};
+  a.rho = h->rho.p;
+  a.elem = sl.elem;
+  a.alpha = sl.alpha;
+  a.scale = sl.scale;
+  a.count = sl.row_off + (int64_t)h->g.ny * h->g.nz;
+  a.grid = 2 * h->num_sms;
+  return h->prec == BIOFVM_FP64 ? launch_src_f64(a, st) : launch_src_f32(a, st);
+}
+
+// Whether the adjoint's steps run on the row-padded working copy as biofvm_step does: their
+// states between the stages are field-shaped arrays, copied out after each solve.
+bool adjoint_pitched(const biofvm *h) { return h->pitched && !h->any_dir && h->n_dnode == 0; }
 
 // `pitched`: the three pipelined sweeps on the row-padded working copy (no
 // Dirichlet nodes then).
@@ -2090,7 +2108,7 @@ biofvm_status biofvm_run_stage(biofvm_t *h, int stage) {
     case 1: CK(launch_x(h, kSolve | kDirAfter, st)); CK(launch_nodes(h, st, 0, -1)); break;
     case 2: CK(launch_col(h, 1, kSolve | kDirAfter, st)); CK(launch_nodes(h, st, 0, -1)); break;
     case 3: CK(launch_col(h, 2, kSolve | kDirAfter, st)); CK(launch_nodes(h, st, 0, -1)); break;
-    case 4: CK(launch_x(h, kSrc, st)); break;
+    case 4: CK(launch_src(h, st)); break;
     case 5: CK(launch_x(h, kSolve, st)); break;
     case 6: CK(launch_col(h, 1, kSolve, st)); break;
     case 7: CK(launch_col(h, 2, kSolve, st)); break;
@@ -2134,8 +2152,17 @@ biofvm_status biofvm_step_save(biofvm_t *h, void *saved) {
     }
     return launch_nodes(h, st, 0, -1);
   };
-  CK(launch_x(h, kSrc, st));
+  CK(launch_src(h, st));
   CK(cudaMemcpyAsync(sv, h->rho.p, bytes, cudaMemcpyDeviceToDevice, st));
+  if (adjoint_pitched(h)) {
+    CK(pitch_copy(h, true, st));
+    for (int axis = 0; axis < 3; axis++) {
+      CK(launch_pipe(h, axis, kSolve, st, h->prow.p, 0, true));
+      CK(pitch_copy(h, false, st, sv + (axis + 1) * bytes));
+    }
+    CK(cudaMemcpyAsync(h->rho.p, sv + 3 * bytes, bytes, cudaMemcpyDeviceToDevice, st));
+    return BIOFVM_OK;
+  }
   CK(B());
   CK(launch_x(h, kSolve, st));
   CK(cudaMemcpyAsync(sv + bytes, h->rho.p, bytes, cudaMemcpyDeviceToDevice, st));
@@ -2227,17 +2254,26 @@ biofvm_status biofvm_adjoint_step_rates(biofvm_t *h, const void *grad_out, void 
     }
     return launch_nodes(h, st, 0, -1, true, h->adj.p);
   };
-  CK(cudaMemcpyAsync(h->adj.p, grad_out, bytes, cudaMemcpyDeviceToDevice, st));
-  CK(Bt());
-  CK(launch_col(h, 2, kSolve, st, 1));
-  CK(reduce(2, sv + 3 * bytes));
-  CK(Bt());
-  CK(launch_col(h, 1, kSolve, st, 1));
-  CK(reduce(1, sv + 2 * bytes));
-  CK(Bt());
-  CK(launch_x(h, kSolve, st, h->adj.p));
-  CK(reduce(0, sv + bytes));
-  CK(Bt());
+  if (adjoint_pitched(h)) {
+    CK(pitch_copy(h, true, st, const_cast<void *>(grad_out)));
+    for (int axis = 2; axis >= 0; axis--) {
+      CK(launch_pipe(h, axis, kSolve, st, h->prow.p, 0, true));
+      CK(pitch_copy(h, false, st, h->adj.p));
+      CK(reduce(axis, sv + (axis + 1) * bytes));
+    }
+  } else {
+    CK(cudaMemcpyAsync(h->adj.p, grad_out, bytes, cudaMemcpyDeviceToDevice, st));
+    CK(Bt());
+    CK(launch_col(h, 2, kSolve, st, 1));
+    CK(reduce(2, sv + 3 * bytes));
+    CK(Bt());
+    CK(launch_col(h, 1, kSolve, st, 1));
+    CK(reduce(1, sv + 2 * bytes));
+    CK(Bt());
+    CK(launch_x(h, kSolve, st, h->adj.p));
+    CK(reduce(0, sv + bytes));
+    CK(Bt());
+  }
   SrcAdjLaunch a{};
   a.gbar = h->adj.p;
   a.u1 = sv;

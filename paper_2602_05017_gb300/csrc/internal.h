@@ -139,6 +139,15 @@ struct NodeLaunch {
   int S, zero, grid;
 };
 
+// Source update alone: rho[elem[k]] = (rho[elem[k]] + alpha[k]) * scale[k] for k < *count
+// (device); elem unique.
+struct SrcLaunch {
+  void *rho;
+  const int64_t *elem, *count;
+  const void *alpha, *scale;
+  int grid;
+};
+
 struct ReduceLaunch {
   const void *mu, *u;           // adjoint after the sweep, forward sweep output
   long long nel, stride, used;  // elements; element stride along the axis; threads used
@@ -238,6 +247,8 @@ cudaError_t launch_planes_f64(const PlanesArgs &a, int grid, size_t smem, cudaSt
 void set_error_message(const char *msg);
 
 cudaError_t launch_adj_reduce_f64(const ReduceLaunch &a, cudaStream_t st);
+cudaError_t launch_src_f64(const SrcLaunch &a, cudaStream_t st);
+cudaError_t launch_src_f32(const SrcLaunch &a, cudaStream_t st);
 cudaError_t launch_nodes_f64(const NodeLaunch &a, cudaStream_t st);
 cudaError_t launch_nodes_f32(const NodeLaunch &a, cudaStream_t st);
 cudaError_t launch_adj_reduce_f32(const ReduceLaunch &a, cudaStream_t st);

@@ -51,6 +51,10 @@ cudaError_t allow_x_smem_f32(int maxm, size_t bytes) {
 }
 
 
+cudaError_t launch_src_f32(const SrcLaunch &a, cudaStream_t st) {
+  return launch_src_one<float>(a, st);
+}
+
 cudaError_t launch_nodes_f32(const NodeLaunch &a, cudaStream_t st) {
   return launch_nodes_one<float>(a, st);
 }

@@ -44,6 +44,10 @@ cudaError_t allow_x_smem_f64(int maxm, size_t bytes) {
 }
 
 
+cudaError_t launch_src_f64(const SrcLaunch &a, cudaStream_t st) {
+  return launch_src_one<double>(a, st);
+}
+
 cudaError_t launch_nodes_f64(const NodeLaunch &a, cudaStream_t st) {
   return launch_nodes_one<double>(a, st);
 }
