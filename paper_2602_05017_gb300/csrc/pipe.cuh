@@ -146,6 +146,13 @@ __device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
   return r;
 }
 
+// Let the stream's next kernel be scheduled, then wait for the one before this (both no-ops
+// unless the launches ask for programmatic serialisation).
+__device__ __forceinline__ void grid_dependency_sync() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // A thread's two columns of a staged tile, positions ps elements apart.
 //   PAIR: the columns are neighbours (c, c + 1) at an even offset: one access
 //         of two elements per position;
@@ -502,6 +509,10 @@ __global__ void __maxnreg__(pipe_regs(MAXM))
     for (int q = threadIdx.x; q < ntab; q += blockDim.x) tab[q] = __ldg(gT + q);
   }
   __syncthreads();
+  // Launched with programmatic serialisation: everything above ran while the kernel before it
+  // finished; its results are visible from here on.  (The next kernel of the stream may be
+  // scheduled from now on; it waits here in its turn.)
+  grid_dependency_sync();
 
   // x tiles: Src and B before the solve, applied by warp 1 (the preparer) when
   // the launch has one (a.prep_warp: the host sets it exactly when there is a
@@ -890,7 +901,19 @@ cudaError_t launch_pipe_cw(const CUtensorMap &map, const PipeArgs &a, int grid, 
     return cudaSuccess;
   });
   if (!k) return cudaErrorInvalidConfiguration;
-  return cudaLaunchKernel(k, dim3(grid), dim3(threads), args, smem, st);
+  // a.overlap: the launch latency and the staging of the constants overlap the end of the kernel
+  // before.
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = a.overlap ? 1 : 0;
+  return cudaLaunchKernelExC(&cfg, k, args);
 }
 
 template <int MAXM, typename H>

@@ -89,6 +89,7 @@ struct PipeArgs {
   const uint8_t *dir_on;
   const void *dir_val;
   int *status;
+  int overlap;  // host only: launch with programmatic serialisation
 };
 
 }  // namespace bfv
