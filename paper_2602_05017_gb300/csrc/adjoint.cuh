@@ -23,19 +23,78 @@
 
 namespace bfv {
 
-// A float as a double.  The conversion instruction runs on the FP64 pipe (two
-// lanes a clock and SM), which the sums below already fill, so the value is
-// widened by integer instructions: subnormals -- an adjoint field far from its
-// sources is full of them and of zeros -- after a multiplication by 2^64.  Only
-// infinities and NaN take the conversion.
-__device__ __forceinline__ double widen_f64(double v) { return v; }
+// A float as a double by integer instructions (the conversion runs on the FP64
+// pipe, two lanes a clock and SM); infinities and NaN take the conversion.
 __device__ __forceinline__ double widen_f64(float v) {
-  const bool sub = fabsf(v) < 1.17549435e-38f;  // below 2^-126
-  const unsigned b = __float_as_uint(sub ? v * 18446744073709551616.0f : v);
-  const unsigned mag = b & 0x7fffffffu;
-  if (mag >= 0x7f800000u) return (double)v;
-  const unsigned hi = mag == 0u ? 0u : (mag >> 3) + (sub ? 0x34000000u : 0x38000000u);
-  return __hiloint2double((int)((b & 0x80000000u) | hi), (int)(mag << 29));
+  const unsigned b = __float_as_uint(v), mag = b & 0x7fffffffu;
+  if (mag - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((b & 0x80000000u) | ((mag >> 3) + 0x38000000u)),
+                            (int)(mag << 29));
+  return (double)v;
+}
+
+constexpr int kFF = 8;  // elements added in pairs of floats at a time
+
+// Sums of eight products in pairs of floats (hi + lo, Knuth's two-sum and the
+// FMA's exact product error: about 48 bits of the sum of the terms' sizes):
+//   s1 += sum a c,   s2 += sum (b - a)(d - c)
+// where the differences enter as exact pairs as well.  The operands are first
+// scaled by powers of two to a largest size in [1, 2), so that neither the
+// products nor their errors leave the range of a float; the two sums then join
+// FP64 accumulators, four FP64 operations per eight elements.
+__device__ __forceinline__ void ff_two_sum(float &hi, float &lo, float p, float e) {
+  const float s = __fadd_rn(hi, p), t = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(p, t)), e));
+  hi = s;
+}
+__device__ __forceinline__ float ff_two_diff(float x, float y, float &err) {
+  const float s = __fsub_rn(x, y), t = __fsub_rn(s, x);
+  err = __fsub_rn(__fsub_rn(x, __fsub_rn(s, t)), __fadd_rn(y, t));
+  return s;
+}
+// The power of two that brings `top` to [1, 2) (subnormals: as far as one goes), as its exponent.
+__device__ __forceinline__ int ff_exponent(float top) {
+  return min((int)(__float_as_uint(top) >> 23), 253) - 127;
+}
+__device__ __forceinline__ void ff_add(const float (&a)[kFF], const float (&b)[kFF],
+                                       const float (&c)[kFF], const float (&d)[kFF], double &s1,
+                                       double &s2) {
+  float ta = 0.f, tc = 0.f;
+#pragma unroll
+  for (int k = 0; k < kFF; k++) {
+    ta = fmaxf(ta, fmaxf(fabsf(a[k]), fabsf(b[k])));
+    tc = fmaxf(tc, fmaxf(fabsf(c[k]), fabsf(d[k])));
+  }
+  if (fmaxf(ta, tc) == __int_as_float(0x7f800000)) {  // infinities: as FP64 sums them
+#pragma unroll 1
+    for (int k = 0; k < kFF; k++) {
+      float x = 0.f, y = 0.f, z = 0.f, w = 0.f;
+#pragma unroll
+      for (int j = 0; j < kFF; j++)
+        if (j == k) x = a[j], y = b[j], z = c[j], w = d[j];
+      s1 = fma((double)x, (double)z, s1);
+      s2 = fma((double)y - (double)x, (double)w - (double)z, s2);
+    }
+    return;
+  }
+  const int ea = ff_exponent(ta), ec = ff_exponent(tc);
+  const float fa = __uint_as_float((unsigned)(127 - ea) << 23);
+  const float fc = __uint_as_float((unsigned)(127 - ec) << 23);
+  float h1 = 0.f, l1 = 0.f, h2 = 0.f, l2 = 0.f;
+#pragma unroll
+  for (int k = 0; k < kFF; k++) {
+    const float x = __fmul_rn(a[k], fa), y = __fmul_rn(c[k], fc);
+    float p = __fmul_rn(x, y);
+    ff_two_sum(h1, l1, p, __fmaf_rn(x, y, -p));
+    float de, df;
+    const float dx = ff_two_diff(__fmul_rn(b[k], fa), x, de);
+    const float dy = ff_two_diff(__fmul_rn(d[k], fc), y, df);
+    p = __fmul_rn(dx, dy);
+    ff_two_sum(h2, l2, p, __fmaf_rn(de, dy, __fmaf_rn(dx, df, __fmaf_rn(dx, dy, -p))));
+  }
+  const double scale = __hiloint2double((1023 + ea + ec) << 20, 0);
+  s1 = fma(widen_f64(h1) + widen_f64(l1), scale, s1);
+  s2 = fma(widen_f64(h2) + widen_f64(l2), scale, s2);
 }
 
 // Positions of a line one thread walks at a time.
@@ -47,9 +106,11 @@ constexpr int kReduceSeg = 32;
 //   y, z: an item is kReduceSeg consecutive positions of one line (neighbouring
 //         threads take neighbouring lines), each element read and widened once;
 //   x:    an item is one element; its neighbour S further on is the next lanes'.
-// Bound by its four FP64 operations per element (4.2M elements: 29 us at the
-// measured FP64 rate).  One element per item with a 64-bit division each and two
-// conversions more took 45 us (FP64 fields) and 72 us (FP32).
+// FP64 fields are bound by their four FP64 operations per element (4.2M
+// elements: 29 us at the measured FP64 rate; one element per item with a 64-bit
+// division each took 45).  FP32 fields sum eight elements at a time in pairs of
+// floats first (ff_add): 4M elements in about 19 us, against 50 with every element
+// widened to FP64 and 72 with the division and four conversions as well.
 // partial layout: [block][2][S].
 template <typename E>
 __global__ void __launch_bounds__(kReduceThreads)
@@ -62,14 +123,27 @@ __global__ void __launch_bounds__(kReduceThreads)
     const long long rowlen = (long long)n_axis * S;
     const long long step = used % rowlen;
     long long at = tid % rowlen;  // the element's place in its row
-#pragma unroll 4
-    for (long long e = tid; e < nel; e += used) {
-      const double m0 = widen_f64(mu[e]), u0 = widen_f64(u[e]);
-      s1 = fma(m0, u0, s1);
-      if (at + S < rowlen)
-        s2 = fma(widen_f64(mu[e + S]) - m0, widen_f64(u[e + S]) - u0, s2);
-      at += step;
-      if (at >= rowlen) at -= rowlen;
+    for (long long e = tid; e < nel;) {
+      E m0[kFF], m1[kFF], u0[kFF], u1[kFF];
+#pragma unroll
+      for (int k = 0; k < kFF; k++, e += used) {
+        const bool ok = e < nel, next = ok && at + S < rowlen;
+        m0[k] = ok ? mu[e] : E(0);
+        u0[k] = ok ? u[e] : E(0);
+        m1[k] = next ? mu[e + S] : m0[k];  // (the last of a line: a zero difference)
+        u1[k] = next ? u[e + S] : u0[k];
+        at += step;
+        if (at >= rowlen) at -= rowlen;
+      }
+      if constexpr (sizeof(E) == 4) {
+        ff_add(m0, m1, u0, u1, s1, s2);
+      } else {
+#pragma unroll
+        for (int k = 0; k < kFF; k++) {
+          s1 = fma(m0[k], u0[k], s1);
+          s2 = fma(m1[k] - m0[k], u1[k] - u0[k], s2);
+        }
+      }
     }
   } else if (tid < used) {
     const long long ncol = nel / n_axis;
@@ -78,33 +152,37 @@ __global__ void __launch_bounds__(kReduceThreads)
       const long long seg = w / ncol, c = w - seg * ncol, plane = c / stride;
       const int i0 = (int)seg * kReduceSeg, i1 = min(n_axis, i0 + kReduceSeg);
       long long e = (plane * n_axis + i0) * stride + (c - plane * stride);
-      double m0 = widen_f64(mu[e]), u0 = widen_f64(u[e]);
-      int i = i0 + 1;
-      for (; i + 8 <= i1; i += 8) {
-        E mb[8], ub[8];
+      E mp = mu[e], up = u[e];
+      for (int i = i0; i < i1; i += kFF) {  // positions i .. i+7 and the one after each
+        E m0[kFF], m1[kFF], u0[kFF], u1[kFF];
 #pragma unroll
-        for (int k = 0; k < 8; k++) {
-          mb[k] = mu[e + (k + 1) * stride];
-          ub[k] = u[e + (k + 1) * stride];
+        for (int k = 0; k < kFF; k++) {
+          const bool ok = i + k < i1, next = ok && i + k + 1 < n_axis;
+          m1[k] = next ? mu[e + (k + 1) * stride] : E(0);
+          u1[k] = next ? u[e + (k + 1) * stride] : E(0);
         }
-        e += 8 * stride;
+        e += kFF * stride;
 #pragma unroll
-        for (int k = 0; k < 8; k++) {
-          const double m1 = widen_f64(mb[k]), u1 = widen_f64(ub[k]);
-          s1 = fma(m0, u0, s1);
-          s2 = fma(m1 - m0, u1 - u0, s2);
-          m0 = m1;
-          u0 = u1;
+        for (int k = 0; k < kFF; k++) {
+          const bool ok = i + k < i1, next = ok && i + k + 1 < n_axis;
+          m0[k] = ok ? mp : E(0);
+          u0[k] = ok ? up : E(0);
+          mp = m1[k];
+          up = u1[k];
+          if (!next) {  // the line's last position (or none): a zero difference
+            m1[k] = m0[k];
+            u1[k] = u0[k];
+          }
         }
-      }
-      for (; i <= i1; i++) {  // the rest, and the difference to the next segment's first position
-        s1 = fma(m0, u0, s1);
-        if (i == n_axis) break;
-        e += stride;
-        const double m1 = widen_f64(mu[e]), u1 = widen_f64(u[e]);
-        s2 = fma(m1 - m0, u1 - u0, s2);
-        m0 = m1;
-        u0 = u1;
+        if constexpr (sizeof(E) == 4) {
+          ff_add(m0, m1, u0, u1, s1, s2);
+        } else {
+#pragma unroll
+          for (int k = 0; k < kFF; k++) {
+            s1 = fma(m0[k], u0[k], s1);
+            s2 = fma(m1[k] - m0[k], u1[k] - u0[k], s2);
+          }
+        }
       }
     }
   }
