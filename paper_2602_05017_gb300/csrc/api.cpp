@@ -153,7 +153,7 @@ struct biofvm {
   int small_T[3] = {1, 1, 1}, small_m[3] = {1, 1, 1};  // chunks per axis of the small step
   DevBuf small_tab[3];                                   // their tables (LineTab; small_planes: axis_tables)
   int pipe_chunk = 0;        // FP32 pipelined sweeps: chunk length (0: the planner's)
-  int pipe_cw = 0;           // FP32 pipelined sweeps: lines per tile, 32 or 16 (0: the planner's)
+  int pipe_cw = 0;           // FP32 pipelined sweeps: lines per tile, 32, 24 or 16 (0: the planner's)
   int pipe_ns = 4;           // FP32 pipelined sweeps: most ring stages per CTA
   DevBuf scratch;            // FP32 streaming: forward intermediate, field-sized
   int forced = 0;  // chunk lengths fixed by the caller (batched environments)
@@ -506,8 +506,8 @@ int x_tile_wavefronts(int64_t pitch, int S, int cw, int m, size_t esz) {
 // Plan the pipelined sweep of axis 0 (x), 1 (y) or 2 (z) over `field`, whose
 // rows (nx*S elements) start gp elements apart; leaves p.use = 0 when the plain
 // kernels have to be used instead.  Tiles of 32 columns when a ring of >= 2
-// stages of them fits in shared memory with the constants, else tiles of 16
-// columns (long lines; two chunks per consumer warp).
+// stages of them fits in shared memory with the constants, else tiles of 24
+// (y, z) or 16 columns (long lines).
 void plan_pipe(biofvm *h, int axis, PipePlan &p, int64_t gp, void *field) {
   p = PipePlan{};
   const int64_t nx = h->g.nx, ny = h->g.ny, nz = h->g.nz, S = h->g.n_sub;
@@ -1360,7 +1360,10 @@ biofvm_status build_sources(biofvm *h) {
   std::vector<int64_t> order(n), tmp(n);
   for (int64_t k = 0; k < n; k++) order[k] = k;
   const int64_t nvox = (int64_t)h->g.nx * h->g.ny * h->g.nz;
-  for (int shift = 0; shift < 63 && ((nvox - 1) >> shift) > 0; shift += 11) {
+  if (n <= 512)  // (few agents: counting 2048 digits costs more than comparing)
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int64_t i, int64_t j) { return h->h_voxel[i] < h->h_voxel[j]; });
+  for (int shift = 0; n > 512 && shift < 63 && ((nvox - 1) >> shift) > 0; shift += 11) {
     int64_t at[2049] = {0};
     auto digit = [&](int64_t k) { return (h->h_voxel[k] >> shift) & 2047; };
     for (int64_t k = 0; k < n; k++) at[digit(k) + 1]++;

@@ -30,8 +30,8 @@
 // 0.51 ms a sweep at 400^3 x 4 (4.0 TB/s).  Pairs halve the instructions,
 // chunks whose coefficients have reached their interior values (all but the
 // first one or two and the last of a line) read none, and running the
-// recurrences again from the true carry replaces the correction passes: about
-// six instructions per element.  Chunks are short (16 positions) because the
+// recurrences again from the true carry replaces the correction passes: 16
+// instructions per element, all warps of the CTA counted.  Chunks are short (16 positions) because the
 // four dependent chains per tile are the remaining latency.  Measured, x / y /
 // z of 400^3 x 4: 0.540 / 0.506 / 0.513 ms before, 0.34 / 0.33 / 0.39 after
 // (HBM copy rate: 0.306); the z sweep's rows are 128 bytes, a plane apart.
