@@ -252,7 +252,8 @@ int biofvm_launches_per_step(const biofvm_t *h);
  * line written to the host buffer out[len]: "cooperative" (small FP64 grids:
  * all steps of a call in one launch), or "x=K y=K z=K" with K one of stream
  * (whole-line streaming sweep), pipe (TMA-pipelined tiles, followed by
- * "/cwC/mM": C lines per tile, chunks of M positions) or plain (register-chunk
+ * "/cwC/mM": C lines per tile, chunks of M positions, and "/split" when their
+ * coefficients are staged per substrate) or plain (register-chunk
  * kernels), then " scaled" when the FP64 steps carry the renormalisation
  * factor, " pitched" when the steps run on a row-padded copy of the field (an
  * FP32 field whose rows of nx*n_sub elements are not 16-byte multiples,

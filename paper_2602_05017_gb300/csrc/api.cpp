@@ -23,6 +23,7 @@
 #include "agents.h"
 #include "batch_args.h"
 #include "pipe_args.h"
+#include "pipe_plan.h"
 #include "internal.h"
 
 using namespace bfv;
@@ -77,13 +78,8 @@ struct ColPlan {
 // Persistent TMA pipeline of one FP32 sweep (used when rows are 16-byte aligned
 // and a ring of >= 2 stages with the constants fits in shared memory; otherwise
 // the plain kernels).
-struct PipePlan {
-  int use = 0, T = 1, m = 1, maxm = 8;
-  int cw = 32, W = 1;  // columns per tile (32, or 24 or 16 for long lines); consumer warps
-  int box_rows = 0, nbox = 0, rows_per_tile = 0, pitch = 0;
-  int stages = 0, ctas = 1, grid = 0;  // ctas: per SM
-  int64_t stage_elems = 0, ntiles = 0;
-  size_t smem = 0;
+struct PipePlan : PipeShape {
+  int use = 0, grid = 0;
   CUtensorMap map[2]{};  // y/z: [0] the field, [1] the adjoint field
   int have_map[2]{};
 };
@@ -152,9 +148,7 @@ struct biofvm {
   DevBuf small_bar;
   int small_T[3] = {1, 1, 1}, small_m[3] = {1, 1, 1};  // chunks per axis of the small step
   DevBuf small_tab[3];                                   // their tables (LineTab; small_planes: axis_tables)
-  int pipe_chunk = 0;        // FP32 pipelined sweeps: chunk length (0: the planner's)
-  int pipe_cw = 0;           // FP32 pipelined sweeps: lines per tile, 32, 24 or 16 (0: the planner's)
-  int pipe_ns = 4;           // FP32 pipelined sweeps: most ring stages per CTA
+  PipeKnobs pipe_knobs;      // pipelined sweeps
   DevBuf scratch;            // FP32 streaming: forward intermediate, field-sized
   int forced = 0;  // chunk lengths fixed by the caller (batched environments)
   int batched = 0;  // an environment of a batch in per-environment mode
@@ -473,130 +467,13 @@ bool encode_pipe_map(biofvm *h, PipePlan &p, int axis, int buf, void *field, int
   return p.have_map[buf] != 0;
 }
 
-// Shared-memory wavefronts of one warp access of the pipelined x tile at row
-// pitch `pitch` (elements): lane l reads column pair l % (cw/2) of its chunk, m
-// positions from the next lane group's, as pipe.cuh does -- S = 1: four
-// consecutive positions of a row, S = 2: two positions of both substrates, even
-// S: a pair of substrates, else one column.  The hardware serves 128 bytes of
-// lanes at a time; a group of lanes costs the most distinct words in one bank.
-int x_tile_wavefronts(int64_t pitch, int S, int cw, int m, size_t esz) {
-  const bool wide = S == 1 || S == 2;
-  const bool even = S == 2 || S == 4 || S == 8;
-  const int width = (int)esz * (wide ? 4 : even ? 2 : 1);  // bytes a lane reads
-  const int pw = cw / 2, per = std::max(1, std::min(32, 128 / width)), ncol = cw / S * S;
-  int total = 0;
-  for (int g = 0; g < 32; g += per) {
-    std::vector<int64_t> words[32];
-    size_t worst = 0;
-    for (int l = g; l < std::min(32, g + per); l++) {
-      int c = S == 1 ? l % pw : 2 * (l % pw);
-      if (c >= ncol) c = 0;
-      const int64_t byte = ((c / S) * pitch + c % S + (int64_t)(l / pw) * m * S) * (int64_t)esz;
-      for (int64_t w = byte / 4; w <= (byte + width - 1) / 4; w++) {
-        std::vector<int64_t> &v = words[w & 31];
-        if (std::find(v.begin(), v.end(), w) == v.end()) v.push_back(w);
-        worst = std::max(worst, v.size());
-      }
-    }
-    total += (int)worst;
-  }
-  return total;
-}
-
 // Plan the pipelined sweep of axis 0 (x), 1 (y) or 2 (z) over `field`, whose
 // rows (nx*S elements) start gp elements apart; leaves p.use = 0 when the plain
-// kernels have to be used instead.  Tiles of 32 columns when a ring of >= 2
-// stages of them fits in shared memory with the constants, else tiles of 24
-// (y, z) or 16 columns (long lines).
+// kernels have to be used instead.
 void plan_pipe(biofvm *h, int axis, PipePlan &p, int64_t gp, void *field) {
   p = PipePlan{};
-  const int64_t nx = h->g.nx, ny = h->g.ny, nz = h->g.nz, S = h->g.n_sub;
-  const size_t esz = h->esz;
-  const int n = axis_len(h, axis);
   if (h->prec == BIOFVM_FP64) return;  // FP64 streams whole lines instead
-  for (int cw : {32, 24, 16}) {
-    if (h->pipe_cw && cw != h->pipe_cw) continue;
-    if (cw == 24 && axis == 0) continue;
-    PipePlan q{};
-    q.cw = cw;
-    const int cpw = pipe_chunks_per_warp(cw);
-    const int extra = axis == 0 ? 2 : 1;  // warps besides the consumers: producer (+ preparer)
-    // chunks of exactly the capacity (the last one shorter; positions past the line's end have
-    // zero coefficients), the shortest whose warps fit in a CTA.  48 positions (y/z) keep long
-    // lines on tiles of 32 or 24 columns: z sweeps read one tile row per plane, and with 16
-    // columns, 64 bytes, a 1200 x 400 x 900 x 2 sweep ran at 2.5 TB/s (with 24 at 3.7).
-    bool found = false;
-    for (int target : {16, 24, 48}) {
-      const int want = h->pipe_chunk > 0 ? h->pipe_chunk : target;
-      q.m = q.maxm = want <= 8 && cw == 32 ? 8 : want <= 16 ? 16 : want <= 24 ? 24 : 48;
-      if (q.maxm == 48 ? axis == 0 || cw == 16 : cw == 24) continue;
-      q.T = (n + q.m - 1) / q.m;
-      q.W = (q.T + cpw - 1) / cpw;
-      if (q.W + extra > pipe_sm_warps(q.maxm)) continue;
-      found = true;
-      break;
-    }
-    if (!found) continue;
-    if (axis == 0) {
-      if ((gp * (int64_t)esz) % 16 != 0 || S > cw) continue;
-      q.rows_per_tile = (int)(cw / S);
-      // the staged rows: gp elements each (a 16-byte multiple), at a shared-memory pitch in
-      // elements that keeps every row 16-byte aligned
-      const int align = (int)(16 / esz);
-      int best = 1 << 30;
-      for (int64_t pitch = gp; pitch <= gp + 64; pitch += align) {
-        const int d = x_tile_wavefronts(pitch, (int)S, cw, q.m, esz);
-        if (d < best) {
-          best = d;
-          q.pitch = (int)pitch;
-        }
-      }
-      q.stage_elems = (int64_t)q.rows_per_tile * q.pitch;
-      if (ny * nz > (int64_t)0x7fffffff) return;  // the kernel tracks rows in 32 bits
-      q.ntiles = (ny * nz + q.rows_per_tile - 1) / q.rows_per_tile;
-    } else {
-      const int64_t C = axis == 1 ? nx * S : ny * gp;
-      const int nplanes = axis == 1 ? (int)nz : 1;
-      // the map's stride between a line's positions must be a 16-byte multiple: y: the row
-      // pitch gp; z: the plane, C = ny * gp (the inner extent C of a y map need not be)
-      const int64_t lstride = axis == 1 ? gp : C;
-      if ((lstride * (int64_t)esz) % 16 != 0 || C > (int64_t)0x7fffffff || nplanes > 65535)
-        return;
-      // boxes of at most 256 rows; a tensor copy's shared-memory destination must be
-      // 128-byte aligned, so box_rows * cw * esz is rounded up to a 128-byte multiple (rows
-      // past the line's end are filled with zeros on load and skipped on store)
-      q.nbox = (n + 255) / 256;
-      const int rgran = cw == 24 ? (int)(16 / esz) : std::max(1, (int)(128 / ((size_t)cw * esz)));
-      q.box_rows = ((n + q.nbox - 1) / q.nbox + rgran - 1) / rgran * rgran;
-      if (((size_t)q.box_rows * cw * esz) % 128 != 0 || q.box_rows > 256) continue;
-      q.stage_elems = (int64_t)q.nbox * q.box_rows * cw;
-      q.ntiles = (int64_t)nplanes * ((C + cw - 1) / cw);
-      if (q.ntiles > (int64_t)0x7fffffff) return;  // tiles are indexed in 32 bits
-    }
-    const size_t stage = (size_t)q.stage_elems * esz;
-    const size_t tab = (size_t)pipe_tab_pairs(q.maxm, (int)S, q.W, cpw) * 8 + 16;  // + alignment
-    // carry exchange [2][W][32 / cpw] pairs; mbarriers: full, done, ready per stage, at most 8 stages
-    const size_t scratch = 2 * (size_t)q.W * (32 / cpw) * 8 + 3 * 8 * 8;
-    // As many CTAs per SM as the registers take, while each keeps three stages (256 positions:
-    // two CTAs of 9 warps); else one with as many stages as fit.
-    const int most = std::max(2, std::min(h->pipe_ns, 8));
-    for (int c = std::max(1, pipe_sm_warps(q.maxm) / (q.W + extra)); c >= 1 && !q.stages; c--) {
-      const size_t room = std::min(kMaxDynamicSmem, (kMaxDynamicSmem + 1024) / c - 1024);
-      for (int ns = most; ns >= (c > 1 ? std::min(3, most) : 2) && !q.stages; ns--)
-        if (ns * stage + tab + scratch <= room) {
-          q.stages = ns;
-          q.ctas = c;
-        }
-    }
-    if (!q.stages) continue;
-    q.smem = q.stages * stage + tab + scratch;
-    p = q;
-    break;
-  }
-  if (!p.stages) {
-    p = PipePlan{};
-    return;
-  }
+  if (!pipe_shape(axis, h->g.nx, h->g.ny, h->g.nz, h->g.n_sub, h->esz, gp, h->pipe_knobs, p)) return;
   if (axis != 0 && !encode_pipe_map(h, p, axis, 0, field, gp)) {
     p.use = 0;
     return;
@@ -872,13 +749,13 @@ biofvm_status upload_constants(biofvm *h) {
     if (st) return st;
     if (f32)
       stream_consts_f32(h, axis, t, &c32[(size_t)axis * 2 * h->g.n_sub], h->stream_k0[axis]);
-    // the pipelined kernel's constants as pairs of substrates (pipe_args.h: pipe_tab_pairs)
+    // the pipelined kernel's constants (pipe_args.h: pipe_tab_pairs)
     auto upload_T = [&](DevBuf &dst, const PipePlan &q) -> biofvm_status {
       if (!q.use) return BIOFVM_OK;
       const int n = axis_len(h, axis), S = h->g.n_sub;
       const int ncls = pipe_classes(S), cpw = pipe_chunks_per_warp(q.cw), nch = q.W * cpw;
       const int npad = pipe_npad(nch * q.maxm);
-      std::vector<double> tt((size_t)2 * pipe_tab_pairs(q.maxm, S, q.W, cpw), 0.0);
+      std::vector<double> tt((size_t)2 * pipe_tab_pairs(q.maxm, S, q.W, cpw, q.split), 0.0);
       const double *inv = t.data(), *mul = inv + (size_t)n * S;
       const double *pc = mul + 3 * (size_t)n * S;
       for (int c = 0; c < ncls; c++)
@@ -892,10 +769,15 @@ biofvm_status upload_constants(biofvm *h) {
           put((size_t)4 * c + 3, cfix[S + s]);
           const size_t p0 = (size_t)4 * ncls;
           for (int i = 0; i < n; i++) {
-            put(p0 + (size_t)c * npad + i, inv[(size_t)i * S + s]);
-            put(p0 + ((size_t)ncls + c) * npad + i, mul[(size_t)i * S + s]);
+            if (q.split) {  // per substrate (every one is the first of its class)
+              tt[2 * p0 + (size_t)s * npad + i] = inv[(size_t)i * S + s];
+              tt[2 * p0 + ((size_t)S + s) * npad + i] = mul[(size_t)i * S + s];
+            } else {
+              put(p0 + (size_t)c * npad + i, inv[(size_t)i * S + s]);
+              put(p0 + ((size_t)ncls + c) * npad + i, mul[(size_t)i * S + s]);
+            }
           }
-          const size_t p1 = p0 + (size_t)2 * ncls * npad, p2 = p1 + (size_t)ncls * nch * kWtN;
+          const size_t p1 = p0 + (size_t)(q.split ? S : 2 * ncls) * npad, p2 = p1 + (size_t)ncls * nch * kWtN;
           for (int j = 0; j < nch; j++) {
             const int w = j / cpw;
             // product over chunks lo..hi within warp w
@@ -1072,6 +954,7 @@ cudaError_t launch_pipe(const biofvm *h, int axis, int flags, cudaStream_t st, v
   b.ntiles = p.ntiles;
   b.C = axis == 1 ? (int64_t)h->g.nx * h->g.n_sub : (int64_t)h->g.ny * gp;
   b.cw = p.cw;
+  b.split = p.split;
   b.tiles_per_plane = (int)((b.C + p.cw - 1) / p.cw);
   b.nplanes = axis == 1 ? h->g.nz : 1;
   b.box_rows = p.box_rows;
@@ -1628,9 +1511,9 @@ biofvm_status create_impl(const biofvm_grid *grid, double dx, double dt, const d
   h->num_sms = prop.multiProcessorCount;
   // sweep selection and tuning knobs (environment, read once per handle)
   if (const char *env = getenv("BIOFVM_PIPELINE")) h->pipe_enabled = atoi(env) != 0;
-  if (const char *env = getenv("BIOFVM_PIPE_CHUNK")) h->pipe_chunk = atoi(env);
-  if (const char *env = getenv("BIOFVM_PIPE_CW")) h->pipe_cw = atoi(env);
-  if (const char *env = getenv("BIOFVM_PIPE_NS")) h->pipe_ns = atoi(env);
+  if (const char *env = getenv("BIOFVM_PIPE_CHUNK")) h->pipe_knobs.chunk = atoi(env);
+  if (const char *env = getenv("BIOFVM_PIPE_CW")) h->pipe_knobs.cw = atoi(env);
+  if (const char *env = getenv("BIOFVM_PIPE_NS")) h->pipe_knobs.ns = atoi(env);
   if (const char *env = getenv("BIOFVM_STREAM")) h->stream_enabled = atoi(env) != 0;
   if (const char *env = getenv("BIOFVM_STREAM_CTAS")) h->stream_ctas_per_sm = atoi(env);
   if (const char *env = getenv("BIOFVM_STREAM32")) h->stream32_enabled = atoi(env) != 0;
@@ -1733,7 +1616,7 @@ biofvm_status biofvm_describe(const biofvm_t *h, char *out, size_t len) {
         d += "stream";
       } else if (p.use) {
         char b[48];
-        snprintf(b, sizeof b, "pipe/cw%d/m%d", p.cw, p.m);
+        snprintf(b, sizeof b, "pipe/cw%d/m%d%s", p.cw, p.m, p.split ? "/split" : "");
         d += b;
       } else {
         d += "plain";

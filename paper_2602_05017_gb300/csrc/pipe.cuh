@@ -260,13 +260,40 @@ struct ColPair {
   }
 };
 
-// A chunk pair's constants in shared memory (pipe_args.h).
-struct PairCoef {
-  const f2 *K;                // interior inv' and mul; c_hi, c_lo
-  const ulonglong2 *Ti, *Tm;  // inv' and mul of the chunk's positions, two at a time (0 past the
-                              // line's end)
-  const f2 *wt;               // the chunk's carry weights (kWt*)
-  const f2 *pw;               // [W] products of mul over each warp's chunks
+// A chunk pair's constants in shared memory (pipe_args.h).  inv(i), mul(i): inv' and mul of the
+// chunk's positions i and i + 1, i even (0 past the line's end).
+struct PairCoefBase {
+  const f2 *K;   // interior inv' and mul; c_hi, c_lo
+  const f2 *wt;  // the chunk's carry weights (kWt*)
+  const f2 *pw;  // [W] products of mul over each warp's chunks
+};
+template <bool SPLIT>
+struct PairCoef : PairCoefBase {
+  const ulonglong2 *Ti, *Tm;
+  __device__ __forceinline__ void at(const f2 *tab, int ncls, int npad, int cls, int, int, int lo) {
+    Ti = reinterpret_cast<const ulonglong2 *>(tab + cls * npad + lo);
+    Tm = reinterpret_cast<const ulonglong2 *>(tab + (ncls + cls) * npad + lo);
+  }
+  __device__ __forceinline__ ulonglong2 inv(int i) const { return Ti[i / 2]; }
+  __device__ __forceinline__ ulonglong2 mul(int i) const { return Tm[i / 2]; }
+};
+// Each substrate's coefficients on their own (odd S, where the pairs would not fit).
+template <>
+struct PairCoef<true> : PairCoefBase {
+  const float *Ti0, *Ti1, *Tm0, *Tm1;  // of the pair's two substrates
+  __device__ __forceinline__ void at(const f2 *tab, int ncls, int npad, int, int sa, int sb, int lo) {
+    const float *const t = reinterpret_cast<const float *>(tab);
+    Ti0 = t + sa * npad + lo;
+    Ti1 = t + sb * npad + lo;
+    Tm0 = Ti0 + ncls * npad;  // (ncls == S)
+    Tm1 = Ti1 + ncls * npad;
+  }
+  static __device__ __forceinline__ ulonglong2 two(const float *a, const float *b) {
+    const float2 x = *reinterpret_cast<const float2 *>(a), y = *reinterpret_cast<const float2 *>(b);
+    return make_ulonglong2(f2_pack(x.x, y.x), f2_pack(x.y, y.y));
+  }
+  __device__ __forceinline__ ulonglong2 inv(int i) const { return two(Ti0 + i, Ti1 + i); }
+  __device__ __forceinline__ ulonglong2 mul(int i) const { return two(Tm0 + i, Tm1 + i); }
 };
 // What a thread does with the Dirichlet application after the solve.
 struct PairDir {
@@ -310,10 +337,10 @@ __device__ __forceinline__ f2 scan_bwd(f2 B, int q, const f2 *wt) {
 // kFull: MAXM positions, coefficients from the tables; kRagged: any chunk.
 // Returns false when a consumer's wait for the tile timed out.
 enum { kInner, kFull, kRagged };
-template <int MAXM, int KIND, int CPW, int VEC, typename Cols>
+template <int MAXM, int KIND, int CPW, int VEC, typename Cols, typename Coef>
 __device__ __forceinline__ bool pipe_chunk(const Cols col, const int len, const int lo,
                                            const int n, const int wc, const int W, const int q,
-                                           const int p, const PairCoef &cf, f2 *s_end,
+                                           const int p, const Coef &cf, f2 *s_end,
                                            f2 *s_beg, const int ncons, const PairDir &dir,
                                            const bool st0, const bool st1, const bool ok) {
   constexpr int PW = 32 / CPW;
@@ -354,7 +381,7 @@ __device__ __forceinline__ bool pipe_chunk(const Cols col, const int len, const 
     const f2 after = at(MAXM);
 #pragma unroll
     for (int i = 0; i < MAXM; i += 2) {
-      const ulonglong2 ti = cf.Ti[i / 2], tm = cf.Tm[i / 2];
+      const ulonglong2 ti = cf.inv(i), tm = cf.mul(i);
 #pragma unroll
       for (int k = i; k < i + 2; k++) {
         const f2 a = f2_sub(v[k], k + 1 < MAXM ? v[k + 1] : after);
@@ -390,13 +417,13 @@ __device__ __forceinline__ bool pipe_chunk(const Cols col, const int len, const 
   } else {
 #pragma unroll
     for (int i = 0; i < MAXM; i += 2) {
-      const ulonglong2 tm = cf.Tm[i / 2];
+      const ulonglong2 tm = cf.mul(i);
       v[i] = f2_fma(tm.x, g, v[i]);
       g = v[i + 1] = f2_fma(tm.y, v[i], v[i + 1]);
     }
 #pragma unroll
     for (int i = MAXM - 2; i >= 0; i -= 2) {
-      const ulonglong2 tm = cf.Tm[i / 2];
+      const ulonglong2 tm = cf.mul(i);
       x = f2_fma(tm.x, f2_fma(tm.y, x, v[i + 1]), v[i]);
     }
   }
@@ -441,7 +468,7 @@ __device__ __forceinline__ bool pipe_chunk(const Cols col, const int len, const 
     auto finish = [&](auto dirc) {
 #pragma unroll
       for (int i = MAXM - 2; i >= 0; i -= 2) {
-        const ulonglong2 tm = cf.Tm[i / 2];
+        const ulonglong2 tm = cf.mul(i);
 #pragma unroll
         for (int k = i + 1; k >= i; k--) {
           x = f2_fma(k == i ? tm.x : tm.y, x, v[k]);
@@ -464,7 +491,7 @@ __device__ __forceinline__ bool pipe_chunk(const Cols col, const int len, const 
 // per-access address arithmetic; 0: S read at run time.  CW: columns per tile
 // (32, or 16 for long lines).  H: the field's storage type (E, or bf16 / fp16
 // with E = float): stages and TMA copies hold H, registers and constants E.
-template <int MAXM, int MODE, int PSX = 0, int CW = 32, typename H = float>
+template <int MAXM, int MODE, int PSX = 0, int CW = 32, typename H = float, bool SPLIT = false>
 __global__ void __maxnreg__(pipe_regs(MAXM))
     sweep_pipe_kernel(const __grid_constant__ CUtensorMap map, const PipeArgs a) {
   static_assert(CW == 32 || CW == 24 || CW == 16, "tiles of 32, 24 or 16 columns");
@@ -481,7 +508,7 @@ __global__ void __maxnreg__(pipe_regs(MAXM))
   // array itself (a pointer rounded through an integer would hide from the compiler that what is
   // derived from it lives in shared memory, turning its loads into generic ones)
   f2 *tab = reinterpret_cast<f2 *>(smem_raw + ((size_t)NS * stage_elems * sizeof(H) + 15) / 16 * 16);
-  const int ntab = pipe_tab_pairs(MAXM, S, W, CPW);
+  const int ntab = pipe_tab_pairs(MAXM, S, W, CPW, SPLIT);
   f2 *s_end = tab + ntab;   // [W][PW] warp ends (forward)
   f2 *s_beg = s_end + W * PW;  // [W][PW] warp starts (backward)
   uint64_t *full = reinterpret_cast<uint64_t *>(s_beg + W * PW);
@@ -736,14 +763,13 @@ __global__ void __maxnreg__(pipe_regs(MAXM))
   const int ctid = threadIdx.x - 32 * cons0;  // consumer thread
   long long cn0 = 0, cn1 = 0;                 // entry range of the next tile (dense check)
   if (srcs) tile_range(0, cn0, cn1);
-  PairCoef cf;
+  PairCoef<SPLIT> cf;
   PairDir dir;
   auto set_substrates = [&](int sa, int sb) {
     const int cls = S == 1 ? 0 : S % 2 == 0 ? sa / 2 : sa;
     cf.K = tab + cls * 4;
-    cf.Ti = reinterpret_cast<const ulonglong2 *>(tab + 4 * ncls + cls * npad + lo);
-    cf.Tm = reinterpret_cast<const ulonglong2 *>(tab + 4 * ncls + (ncls + cls) * npad + lo);
-    const f2 *w = tab + 4 * ncls + 2 * ncls * npad;
+    cf.at(tab + 4 * ncls, ncls, npad, cls, sa, sb, lo);
+    const f2 *w = tab + 4 * ncls + (SPLIT ? 1 : 2) * ncls * npad;
     cf.wt = w + (cls * (W * CPW) + t) * kWtN;
     cf.pw = w + ncls * (W * CPW) * kWtN + cls * W;
     dir.on0 = dir_after && a.dir_on[sa];
@@ -873,6 +899,13 @@ cudaError_t pipe_kernels(F &&f) {  // f(x kernel for S, S), ..., f(y/z kernel, -
   }
   return e;
 }
+// The tiles of `split` coefficients (odd S).
+template <int CW, typename H, typename F>
+cudaError_t pipe_split_kernels(F &&f) {
+  const cudaError_t e = f((const void *)sweep_pipe_kernel<kSplitMaxm, 1, 0, CW, H, true>, -1);
+  return e != cudaSuccess ? e
+                          : f((const void *)sweep_pipe_kernel<kSplitMaxm, 0, 0, CW, H, true>, 0);
+}
 // The second tile width of a capacity (0: none).
 constexpr int pipe_narrow(int maxm) { return maxm <= 8 ? 0 : maxm <= 24 ? 16 : 24; }
 
@@ -884,6 +917,10 @@ cudaError_t allow_pipe_smem(size_t bytes) {
   cudaError_t e = pipe_kernels<MAXM, 32, H>(set);
   if constexpr (pipe_narrow(MAXM) > 0)
     if (e == cudaSuccess) e = pipe_kernels<MAXM, pipe_narrow(MAXM), H>(set);
+  if constexpr (MAXM == kSplitMaxm) {
+    if (e == cudaSuccess) e = pipe_split_kernels<32, H>(set);
+    if (e == cudaSuccess) e = pipe_split_kernels<16, H>(set);
+  }
   return e;
 }
 
@@ -896,10 +933,16 @@ cudaError_t launch_pipe_cw(const CUtensorMap &map, const PipeArgs &a, int grid, 
   const int psx = (a.S == 1 || a.S == 2 || a.S == 4 || a.S == 8) ? a.S : 0;
   void *args[] = {const_cast<CUtensorMap *>(&map), const_cast<PipeArgs *>(&a)};
   const void *k = nullptr;
-  pipe_kernels<MAXM, CW, H>([&](const void *f, int s) {
-    if (s == (a.mode != 0 ? -1 : psx)) k = f;
+  const int want = a.mode != 0 ? -1 : psx;
+  auto pick = [&](const void *f, int s) {
+    if (s == want) k = f;
     return cudaSuccess;
-  });
+  };
+  if (a.split) {
+    if constexpr (MAXM == kSplitMaxm) pipe_split_kernels<CW, H>(pick);
+  } else {
+    pipe_kernels<MAXM, CW, H>(pick);
+  }
   if (!k) return cudaErrorInvalidConfiguration;
   // a.overlap: the launch latency and the staging of the constants overlap the end of the kernel
   // before.

@@ -33,7 +33,8 @@ namespace bfv {
 // (2c, 2c+1), S odd: (c, c+1 mod S), S = 1: (0, 0).  AxisTab::tabT holds, in
 // pairs (pipe_tab_pairs of them):
 //   constants   [classes][4]              interior inv' and mul; c_hi, c_lo
-//   inv', mul   [2][classes][npad]        of every position of every chunk (0 past the line)
+//   inv', mul   [2][classes][npad]        of every position of every chunk (0 past the line);
+//               `split` (odd S only): single values [2][S][npad], half as many
 //   weights     [classes][W * chunks per warp][kWtN]  products of mul over whole chunks of
 //               the chunk's warp (1 for chunks past the line):
 //               kWtF0 this chunk; kWtF1 it and the one before; kWtFx all before it;
@@ -52,10 +53,14 @@ BFV_HD constexpr int pipe_classes(int S) { return S > 1 && S % 2 == 0 ? S / 2 : 
 // (two pairs past a multiple of 16: neighbouring classes start in other banks, 16-byte aligned)
 BFV_HD constexpr int pipe_npad(int n) { return (n + 15) / 16 * 16 + 2; }
 // maxm: positions of a chunk.
-BFV_HD constexpr int pipe_tab_pairs(int maxm, int S, int W, int chunks_per_warp) {
-  return pipe_classes(S) * (4 + 2 * pipe_npad(W * chunks_per_warp * maxm) +
+BFV_HD constexpr int pipe_tab_pairs(int maxm, int S, int W, int chunks_per_warp, bool split) {
+  return pipe_classes(S) * (4 + (split ? 1 : 2) * pipe_npad(W * chunks_per_warp * maxm) +
                             W * chunks_per_warp * kWtN + W);
 }
+// The chunk capacity compiled with `split` coefficients (tiles of 32 and 16 columns), for substrate
+// counts whose pairs repeat every coefficient.
+constexpr int kSplitMaxm = 24;
+BFV_HD constexpr bool pipe_can_split(int64_t S) { return S > 1 && S % 2 == 1; }
 // Registers of a thread of chunk capacity maxm (the chunk pair takes 2 maxm): 80, 96, 128 and 168
 // hold the solve with few or no spills, and the warps an SM then has room for (its four register files
 // take whole warps) -- also the largest CTA.
@@ -65,6 +70,7 @@ BFV_HD constexpr int pipe_sm_warps(int maxm) { return 4 * (16384 / (pipe_regs(ma
 struct PipeArgs {
   int mode, n, S, nx, ny, nz;
   int cw;  // columns per tile: 32, 24 or 16
+  int split;
   int64_t ntiles;
   // mode 1 / 2
   int64_t C;

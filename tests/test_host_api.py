@@ -1,0 +1,59 @@
+"""The host half of the library over the stand-in runtime (host_api.py): what it plans, uploads and
+launches."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import host_api
+from paper_2602_05017_gb300 import binding
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    return host_api.load(str(tmp_path_factory.mktemp("host")))
+
+
+# Longest line the pipelined sweep takes for 1 .. 32 substrates with one column per thread and a
+# [T][T][S] table of carry weights, 227 KB of shared memory: (axis > 0, bytes per element).
+LONGEST = {
+    (0, 4): [1280, 1280, 1280, 1155, 1112, 1152, 992, 800, 1018, 906, 768, 704, 640, 608, 576, 544,
+             448, 448, 448, 433, 416, 384, 384, 352, 352, 336, 320, 320, 297, 288, 288, 279],
+    (0, 2): [1280, 1280, 1280, 1280, 1280, 1280, 1280, 1124, 1184, 1088, 992, 800, 752, 704, 672,
+             624, 448, 448, 448, 448, 448, 448, 448, 416, 416, 384, 384, 362, 352, 352, 320, 320],
+    (1, 4): [1408, 1404, 1270, 1152, 1070, 992, 864, 800, 762, 704, 672, 640, 608, 576, 558, 544,
+             512, 500, 480, 452, 448, 428, 416, 416, 384, 384, 380, 352, 352, 352, 320, 320],
+    (1, 2): [1408, 1408, 1408, 1408, 1408, 1344, 1220, 1120, 1040, 864, 816, 768, 736, 684, 640,
+             624, 608, 576, 544, 512, 512, 480, 480, 448, 448, 416, 416, 384, 384, 384, 352, 352],
+}
+
+
+@pytest.mark.parametrize("esz", [4, 2])
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_pipelined_lines_are_no_shorter(lib, axis, esz):
+    out = (ctypes.c_int * 3)()
+    unit = 16 // esz  # elements of a 16-byte row
+    for ns, longest in enumerate(LONGEST[min(axis, 1), esz], 1):
+        for n in {*range(1, longest, 7), *range(max(1, longest - 64), longest + 1)}:
+            dims = [8, 8, 8]
+            dims[axis] = n
+            gp = -(-dims[0] * ns // unit) * unit
+            assert lib.stand_in_pipe_shape(axis, *dims, ns, esz, gp, 0, 0, out), (n, ns)
+
+
+@pytest.mark.parametrize("shape", [(8, 1000, 4, 9), (1272, 8, 4, 7), (8, 8, 448, 25)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_long_16_bit_lines_at_odd_substrate_counts(lib, shape):
+    st, h = host_api.create(lib, *shape, "bf16")
+    assert st == binding.OK
+    assert host_api.describe(lib, h).count("pipe") == 3
+    lib.biofvm_destroy(h)
+
+
+@pytest.mark.parametrize("shape", [(4, 1256, 3, 3), (1072, 4, 4, 5), (4, 8, 1000, 7)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_long_fp32_lines_at_odd_substrate_counts(lib, shape):
+    st, h = host_api.create(lib, *shape, "fp32")
+    assert st == binding.OK
+    assert host_api.describe(lib, h).count("pipe") == 3
+    lib.biofvm_destroy(h)
