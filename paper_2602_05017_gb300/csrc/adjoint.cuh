@@ -56,26 +56,18 @@ __device__ __forceinline__ float ff_two_diff(float x, float y, float &err) {
 __device__ __forceinline__ int ff_exponent(float top) {
   return min((int)(__float_as_uint(top) >> 23), 253) - 127;
 }
+// diff(k): whether element k has a difference (the last of a line has none: b = a, d = c there).
+// A NaN or infinity makes a sum of floats one: the group is then added as FP64 adds it, without
+// the differences that are none (inf - inf there would be NaN).
+template <typename Diff>
 __device__ __forceinline__ void ff_add(const float (&a)[kFF], const float (&b)[kFF],
-                                       const float (&c)[kFF], const float (&d)[kFF], double &s1,
-                                       double &s2) {
+                                       const float (&c)[kFF], const float (&d)[kFF], Diff &&diff,
+                                       double &s1, double &s2) {
   float ta = 0.f, tc = 0.f;
 #pragma unroll
   for (int k = 0; k < kFF; k++) {
     ta = fmaxf(ta, fmaxf(fabsf(a[k]), fabsf(b[k])));
     tc = fmaxf(tc, fmaxf(fabsf(c[k]), fabsf(d[k])));
-  }
-  if (fmaxf(ta, tc) == __int_as_float(0x7f800000)) {  // infinities: as FP64 sums them
-#pragma unroll 1
-    for (int k = 0; k < kFF; k++) {
-      float x = 0.f, y = 0.f, z = 0.f, w = 0.f;
-#pragma unroll
-      for (int j = 0; j < kFF; j++)
-        if (j == k) x = a[j], y = b[j], z = c[j], w = d[j];
-      s1 = fma((double)x, (double)z, s1);
-      s2 = fma((double)y - (double)x, (double)w - (double)z, s2);
-    }
-    return;
   }
   const int ea = ff_exponent(ta), ec = ff_exponent(tc);
   const float fa = __uint_as_float((unsigned)(127 - ea) << 23);
@@ -91,6 +83,18 @@ __device__ __forceinline__ void ff_add(const float (&a)[kFF], const float (&b)[k
     const float dy = ff_two_diff(__fmul_rn(d[k], fc), y, df);
     p = __fmul_rn(dx, dy);
     ff_two_sum(h2, l2, p, __fmaf_rn(de, dy, __fmaf_rn(dx, df, __fmaf_rn(dx, dy, -p))));
+  }
+  if (!(fmaxf(fabsf(h1), fabsf(h2)) <= 3.4e38f) || h1 != h1 || h2 != h2) {
+#pragma unroll 1
+    for (int k = 0; k < kFF; k++) {
+      float x = 0.f, y = 0.f, z = 0.f, w = 0.f;
+#pragma unroll
+      for (int j = 0; j < kFF; j++)
+        if (j == k) x = a[j], y = b[j], z = c[j], w = d[j];
+      s1 = fma((double)x, (double)z, s1);
+      if (diff(k)) s2 = fma((double)y - (double)x, (double)w - (double)z, s2);
+    }
+    return;
   }
   const double scale = __hiloint2double((1023 + ea + ec) << 20, 0);
   s1 = fma(widen_f64(h1) + widen_f64(l1), scale, s1);
@@ -119,29 +123,38 @@ __global__ void __launch_bounds__(kReduceThreads)
   __shared__ double sh[2][kReduceThreads + 32];
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   double s1 = 0.0, s2 = 0.0;
+  // What stands for both ends of a difference that is none: zero (FP64), or the element itself
+  // (FP32, which works on the elements' pairs; ff_add sees to infinities).
+  auto none = [](E v) { return sizeof(E) == 4 ? v : E(0); };
   if (tid < used && stride == S) {  // x
     const long long rowlen = (long long)n_axis * S;
     const long long step = used % rowlen;
     long long at = tid % rowlen;  // the element's place in its row
     for (long long e = tid; e < nel;) {
-      E m0[kFF], m1[kFF], u0[kFF], u1[kFF];
+      E m0[kFF], m1[kFF], u0[kFF], u1[kFF], md[kFF], ud[kFF];
+      const long long at0 = at, e0 = e;
 #pragma unroll
       for (int k = 0; k < kFF; k++, e += used) {
         const bool ok = e < nel, next = ok && at + S < rowlen;
         m0[k] = ok ? mu[e] : E(0);
         u0[k] = ok ? u[e] : E(0);
-        m1[k] = next ? mu[e + S] : m0[k];  // (the last of a line: a zero difference)
-        u1[k] = next ? u[e + S] : u0[k];
+        m1[k] = next ? mu[e + S] : none(m0[k]);
+        u1[k] = next ? u[e + S] : none(u0[k]);
+        md[k] = next ? m0[k] : none(m0[k]);
+        ud[k] = next ? u0[k] : none(u0[k]);
         at += step;
         if (at >= rowlen) at -= rowlen;
       }
       if constexpr (sizeof(E) == 4) {
-        ff_add(m0, m1, u0, u1, s1, s2);
+        auto diff = [&](int k) {
+          return e0 + k * used < nel && (at0 + k * step) % rowlen + S < rowlen;
+        };
+        ff_add(m0, m1, u0, u1, diff, s1, s2);
       } else {
 #pragma unroll
         for (int k = 0; k < kFF; k++) {
           s1 = fma(m0[k], u0[k], s1);
-          s2 = fma(m1[k] - m0[k], u1[k] - u0[k], s2);
+          s2 = fma(m1[k] - md[k], u1[k] - ud[k], s2);
         }
       }
     }
@@ -154,7 +167,7 @@ __global__ void __launch_bounds__(kReduceThreads)
       long long e = (plane * n_axis + i0) * stride + (c - plane * stride);
       E mp = mu[e], up = u[e];
       for (int i = i0; i < i1; i += kFF) {  // positions i .. i+7 and the one after each
-        E m0[kFF], m1[kFF], u0[kFF], u1[kFF];
+        E m0[kFF], m1[kFF], u0[kFF], u1[kFF], md[kFF], ud[kFF];
 #pragma unroll
         for (int k = 0; k < kFF; k++) {
           const bool ok = i + k < i1, next = ok && i + k + 1 < n_axis;
@@ -169,18 +182,21 @@ __global__ void __launch_bounds__(kReduceThreads)
           u0[k] = ok ? up : E(0);
           mp = m1[k];
           up = u1[k];
-          if (!next) {  // the line's last position (or none): a zero difference
-            m1[k] = m0[k];
-            u1[k] = u0[k];
+          md[k] = next ? m0[k] : none(m0[k]);
+          ud[k] = next ? u0[k] : none(u0[k]);
+          if (!next) {  // the line's last position (or none)
+            m1[k] = none(m0[k]);
+            u1[k] = none(u0[k]);
           }
         }
         if constexpr (sizeof(E) == 4) {
-          ff_add(m0, m1, u0, u1, s1, s2);
+          auto diff = [&](int k) { return i + k < i1 && i + k + 1 < n_axis; };
+          ff_add(m0, m1, u0, u1, diff, s1, s2);
         } else {
 #pragma unroll
           for (int k = 0; k < kFF; k++) {
             s1 = fma(m0[k], u0[k], s1);
-            s2 = fma(m1[k] - m0[k], u1[k] - u0[k], s2);
+            s2 = fma(m1[k] - md[k], u1[k] - ud[k], s2);
           }
         }
       }
