@@ -7,9 +7,10 @@
 // (kMaskZero).  For a sweep u = A^-1 d with adjoint mu = A^-1 ubar,
 //     dL/dlambda_s += -(dt/3)      * sum_{elements of s} mu * u
 //     dL/dD_s      += -(dt/dx^2)   * sum_{lines of s} sum_i (mu_{i+1}-mu_i)(u_{i+1}-u_i)
-// (L_N = G^T G with G the first difference).  These sums are reduced in FP64
-// in a fixed order -- per-block partials, then one block over the partials --
-// so repeated runs give bit-identical gradients.
+// (L_N = G^T G with G the first difference).  These sums are reduced to
+// FP64's precision (ff_add for FP32 fields) in a fixed order -- per-block
+// partials, then one block over the partials -- so repeated runs give
+// bit-identical gradients.
 //
 // Src: u1 = (u0 + alpha) / (1 + beta) per element, alpha = sum_k dt w_k S_k
 // rho*_k, beta = sum_k dt w_k (S_k + U_k).  Hence du1/du0 = 1/(1+beta) and,
@@ -33,20 +34,34 @@ __device__ __forceinline__ double widen_f64(float v) {
   return (double)v;
 }
 
-constexpr int kFF = 8;  // elements added in pairs of floats at a time
+constexpr int kFF = 8;  // elements added in floats at a time
 
-// Sums of eight products in pairs of floats (hi + lo, Knuth's two-sum and the
-// FMA's exact product error: about 48 bits of the sum of the terms' sizes):
+// Sums of eight products in floats, to no fewer bits than FP64 gives:
 //   s1 += sum a c,   s2 += sum (b - a)(d - c)
-// where the differences enter as exact pairs as well.  The operands are first
-// scaled by powers of two to a largest size in [1, 2), so that neither the
-// products nor their errors leave the range of a float; the two sums then join
-// FP64 accumulators, four FP64 operations per eight elements.
-__device__ __forceinline__ void ff_two_sum(float &hi, float &lo, float p, float e) {
-  const float s = __fadd_rn(hi, p), t = __fsub_rn(s, hi);
-  lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(p, t)), e));
-  hi = s;
-}
+// Every product and every difference enters as a pair of floats that is exactly it (Knuth's
+// two-sum, the FMA's exact product error), and the pairs are added to three floats (FSum): the sum
+// of the first two is exact, the third collects rounding errors, about 2^-70 of the sum of the
+// terms' sizes.  Per group, FP64 then rounds twice where eight FP64 FMAs round eight times.
+//
+// The operands are scaled by powers of two to a largest size in [1, 2), so nothing overflows.
+// What may be lost at the other end, scaled operands below 2^-149 and products and product
+// errors below it, is less than 2^-142 in either sum, 2^-62 of a sum of at least 2^-80; and it is
+// nothing when the operands' sizes span so little that every product is a multiple of 2^-149.
+// Groups that are neither, or not finite, are added in FP64.
+struct FSum {
+  float h = 0.f, m = 0.f, l = 0.f;
+  static __device__ __forceinline__ float two_sum(float &s, float x) {  // the error
+    const float t = __fadd_rn(s, x), v = __fsub_rn(t, s);
+    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, v)), __fsub_rn(x, v));
+    s = t;
+    return e;
+  }
+  __device__ __forceinline__ void add(float x) { add_small(two_sum(h, x)); }
+  __device__ __forceinline__ void add_small(float x) { l = __fadd_rn(l, two_sum(m, x)); }
+  __device__ __forceinline__ double value() const {
+    return widen_f64(h) + (widen_f64(m) + widen_f64(l));
+  }
+};
 __device__ __forceinline__ float ff_two_diff(float x, float y, float &err) {
   const float s = __fsub_rn(x, y), t = __fsub_rn(s, x);
   err = __fsub_rn(__fsub_rn(x, __fsub_rn(s, t)), __fadd_rn(y, t));
@@ -56,12 +71,12 @@ __device__ __forceinline__ float ff_two_diff(float x, float y, float &err) {
 __device__ __forceinline__ int ff_exponent(float top) {
   return min((int)(__float_as_uint(top) >> 23), 253) - 127;
 }
-// diff(k): whether element k has a difference (the last of a line has none: b = a, d = c there).
-// A NaN or infinity makes a sum of floats one: the group is then added as FP64 adds it, without
-// the differences that are none (inf - inf there would be NaN).
-template <typename Diff>
+// again(k, x, y, z, w): reads element k's a, b, c, d once more (the rare path; keeping them would take
+// 32 registers) and says whether it has a difference (the last of a line has none: b = a, d = c
+// there, but inf - inf would be NaN).
+template <typename Again>
 __device__ __forceinline__ void ff_add(const float (&a)[kFF], const float (&b)[kFF],
-                                       const float (&c)[kFF], const float (&d)[kFF], Diff &&diff,
+                                       const float (&c)[kFF], const float (&d)[kFF], Again &&again,
                                        double &s1, double &s2) {
   float ta = 0.f, tc = 0.f;
 #pragma unroll
@@ -72,33 +87,52 @@ __device__ __forceinline__ void ff_add(const float (&a)[kFF], const float (&b)[k
   const int ea = ff_exponent(ta), ec = ff_exponent(tc);
   const float fa = __uint_as_float((unsigned)(127 - ea) << 23);
   const float fc = __uint_as_float((unsigned)(127 - ec) << 23);
-  float h1 = 0.f, l1 = 0.f, h2 = 0.f, l2 = 0.f;
+  FSum f1, f2;
 #pragma unroll
   for (int k = 0; k < kFF; k++) {
     const float x = __fmul_rn(a[k], fa), y = __fmul_rn(c[k], fc);
     float p = __fmul_rn(x, y);
-    ff_two_sum(h1, l1, p, __fmaf_rn(x, y, -p));
+    f1.add(p);
+    f1.add_small(__fmaf_rn(x, y, -p));
     float de, df;
     const float dx = ff_two_diff(__fmul_rn(b[k], fa), x, de);
     const float dy = ff_two_diff(__fmul_rn(d[k], fc), y, df);
-    p = __fmul_rn(dx, dy);
-    ff_two_sum(h2, l2, p, __fmaf_rn(de, dy, __fmaf_rn(dx, df, __fmaf_rn(dx, dy, -p))));
+    p = __fmul_rn(dx, dy);  // (dx + de)(dy + df), four exact products but for the smallest
+    const float p1 = __fmul_rn(dx, df), p2 = __fmul_rn(de, dy);
+    f2.add(p);
+    f2.add_small(__fmaf_rn(dx, dy, -p));
+    f2.add_small(p1);
+    f2.add_small(p2);
+    f2.l = __fadd_rn(f2.l, __fmaf_rn(de, df, __fadd_rn(__fmaf_rn(dx, df, -p1),
+                                                       __fmaf_rn(de, dy, -p2))));
   }
-  if (!(fmaxf(fabsf(h1), fabsf(h2)) <= 3.4e38f) || h1 != h1 || h2 != h2) {
+  const float least = fminf(fabsf(f1.h), fabsf(f2.h)), most = fabsf(f1.h) + fabsf(f2.h);
+  if (!(least >= 0x1p-80f && most <= 3.4e38f)) {
+    float x, y, z, w;
+    unsigned la = 0xffffffffu, lc = 0xffffffffu;  // smallest sizes - 1: zeros are the largest
+    auto size = [](float v) { return (__float_as_uint(v) & 0x7fffffffu) - 1u; };
 #pragma unroll 1
     for (int k = 0; k < kFF; k++) {
-      float x = 0.f, y = 0.f, z = 0.f, w = 0.f;
-#pragma unroll
-      for (int j = 0; j < kFF; j++)
-        if (j == k) x = a[j], y = b[j], z = c[j], w = d[j];
-      s1 = fma((double)x, (double)z, s1);
-      if (diff(k)) s2 = fma((double)y - (double)x, (double)w - (double)z, s2);
+      again(k, x, y, z, w);
+      la = min(la, min(size(x), size(y)));
+      lc = min(lc, min(size(z), size(w)));
     }
-    return;
+    // binades from the smallest nonzero operands to the largest
+    const int span = (int)(__float_as_uint(ta) >> 23) - max((int)((la + 1u) >> 23), 1) +
+                     (int)(__float_as_uint(tc) >> 23) - max((int)((lc + 1u) >> 23), 1);
+    if (!(most <= 3.4e38f) || span > 103) {
+#pragma unroll 1
+      for (int k = 0; k < kFF; k++) {
+        const bool diff = again(k, x, y, z, w);
+        s1 = fma((double)x, (double)z, s1);
+        if (diff) s2 = fma((double)y - (double)x, (double)w - (double)z, s2);
+      }
+      return;
+    }
   }
   const double scale = __hiloint2double((1023 + ea + ec) << 20, 0);
-  s1 = fma(widen_f64(h1) + widen_f64(l1), scale, s1);
-  s2 = fma(widen_f64(h2) + widen_f64(l2), scale, s2);
+  s1 = fma(f1.value(), scale, s1);
+  s2 = fma(f2.value(), scale, s2);
 }
 
 // Positions of a line one thread walks at a time.
@@ -112,12 +146,13 @@ constexpr int kReduceSeg = 32;
 //   x:    an item is one element; its neighbour S further on is the next lanes'.
 // FP64 fields are bound by their four FP64 operations per element (4.2M
 // elements: 29 us at the measured FP64 rate; one element per item with a 64-bit
-// division each took 45).  FP32 fields sum eight elements at a time in pairs of
-// floats first (ff_add): 4M elements in about 19 us, against 50 with every element
-// widened to FP64 and 72 with the division and four conversions as well.
+// division each took 45).  FP32 fields sum eight elements at a time in three
+// floats first (ff_add): 4.2M elements in 33 us along y and z and 39 along x (FP64 fields 46;
+// pairs of floats, 48 bits, took 24 and 26), bound by the float instructions, about 80 an
+// element.  Every element widened to FP64 took 50, with the division and four conversions 72.
 // partial layout: [block][2][S].
 template <typename E>
-__global__ void __launch_bounds__(kReduceThreads)
+__global__ void __launch_bounds__(kReduceThreads, reduce_blocks_per_sm(sizeof(E)))
     adj_reduce_kernel(const E *__restrict__ mu, const E *__restrict__ u, long long nel, int S,
                       long long stride, int n_axis, long long used, double *__restrict__ partial) {
   __shared__ double sh[2][kReduceThreads + 32];
@@ -146,10 +181,16 @@ __global__ void __launch_bounds__(kReduceThreads)
         if (at >= rowlen) at -= rowlen;
       }
       if constexpr (sizeof(E) == 4) {
-        auto diff = [&](int k) {
-          return e0 + k * used < nel && (at0 + k * step) % rowlen + S < rowlen;
+        auto again = [&](int k, E &x, E &y, E &z, E &w) {
+          const long long ek = e0 + k * used;
+          const bool ok = ek < nel, diff = ok && (at0 + k * step) % rowlen + S < rowlen;
+          x = ok ? mu[ek] : E(0);
+          z = ok ? u[ek] : E(0);
+          y = diff ? mu[ek + S] : x;
+          w = diff ? u[ek + S] : z;
+          return diff;
         };
-        ff_add(m0, m1, u0, u1, diff, s1, s2);
+        ff_add(m0, m1, u0, u1, again, s1, s2);
       } else {
 #pragma unroll
         for (int k = 0; k < kFF; k++) {
@@ -190,8 +231,16 @@ __global__ void __launch_bounds__(kReduceThreads)
           }
         }
         if constexpr (sizeof(E) == 4) {
-          auto diff = [&](int k) { return i + k < i1 && i + k + 1 < n_axis; };
-          ff_add(m0, m1, u0, u1, diff, s1, s2);
+          auto again = [&](int k, E &x, E &y, E &z, E &w) {
+            const long long ek = e + (k - kFF) * stride;
+            const bool ok = i + k < i1, diff = ok && i + k + 1 < n_axis;
+            x = ok ? mu[ek] : E(0);
+            z = ok ? u[ek] : E(0);
+            y = diff ? mu[ek + stride] : x;
+            w = diff ? u[ek + stride] : z;
+            return diff;
+          };
+          ff_add(m0, m1, u0, u1, again, s1, s2);
         } else {
 #pragma unroll
           for (int k = 0; k < kFF; k++) {

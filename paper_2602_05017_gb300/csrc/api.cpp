@@ -2106,7 +2106,7 @@ biofvm_status biofvm_adjoint_step_rates(biofvm_t *h, const void *grad_out, void 
         encode_pipe_map(h, h->pp[axis], axis, 1, h->adj.p, (int64_t)h->g.nx * h->g.n_sub);
   }
   if (!h->partial.p) {
-    h->reduce_blocks = 4 * h->num_sms;
+    h->reduce_blocks = reduce_blocks_per_sm(h->esz) * h->num_sms;
     if (dev_alloc(h->partial, (size_t)h->reduce_blocks * 2 * S * sizeof(double)) != cudaSuccess)
       return fail(BIOFVM_ERR_OOM, "device allocation of the reduction scratch failed");
   }

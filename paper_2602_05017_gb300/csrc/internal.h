@@ -125,8 +125,10 @@ struct PipeArgs;
 // Opt-in dynamic shared memory per CTA on sm_100-class GPUs (227 KB).
 constexpr size_t kMaxDynamicSmem = 232448;
 
-// Threads per block of the adjoint reduction.
+// Threads per block of the adjoint reduction, and the blocks an SM holds at once: 64 registers a
+// thread for FP64 sums, 80 for sums in floats.
 constexpr int kReduceThreads = 256;
+constexpr int reduce_blocks_per_sm(size_t esz) { return esz == 4 ? 3 : 4; }
 
 // Adjoint parameter-gradient reduction of one sweep (adjoint.cuh).
 // Dirichlet nodes: rho[elem[k]] = val[k] * scale[elem[k] % S] (scale NULL: 1),

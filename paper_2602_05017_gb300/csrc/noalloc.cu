@@ -27,6 +27,8 @@
 namespace {
 
 constexpr int kBlocks = 512;
+constexpr int kBlocksF32 = 152 * bfv::reduce_blocks_per_sm(4);  // one wave
+static_assert(kBlocksF32 <= kBlocks, "the scratch holds kBlocks");
 constexpr int kMaxSub = 32;
 constexpr int kMaxDevices = 64;
 
@@ -109,20 +111,21 @@ extern "C" biofvm_status biofvm_param_grad_noalloc(const void *mu, const void *u
   const long long nel = (long long)nx * ny * nz * S;
   const long long stride = axis == 0 ? S : axis == 1 ? (long long)nx * S : (long long)nx * ny * S;
   const int n_axis = axis == 0 ? nx : axis == 1 ? ny : nz;
-  const long long used = (long long)kBlocks * bfv::kReduceThreads / S * S;
+  const int nblocks = prec == BIOFVM_FP64 ? kBlocks : kBlocksF32;
+  const long long used = (long long)nblocks * bfv::kReduceThreads / S * S;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
   if (prec == BIOFVM_FP64) {
-    bfv::adj_reduce_kernel<double><<<kBlocks, bfv::kReduceThreads, 0, st>>>(
+    bfv::adj_reduce_kernel<double><<<nblocks, bfv::kReduceThreads, 0, st>>>(
         static_cast<const double *>(mu), static_cast<const double *>(u), nel, n_sub, stride,
         n_axis, used, partial);
-    bfv::adj_reduce_final_kernel<double><<<1, bfv::kReduceFinalThreads, 0, st>>>(partial, kBlocks, n_sub, -dt / 3.0,
-                                                           -dt / (h_axis * h_axis), dlambda, dD);
+    bfv::adj_reduce_final_kernel<double><<<1, bfv::kReduceFinalThreads, 0, st>>>(
+        partial, nblocks, n_sub, -dt / 3.0, -dt / (h_axis * h_axis), dlambda, dD);
   } else {
-    bfv::adj_reduce_kernel<float><<<kBlocks, bfv::kReduceThreads, 0, st>>>(
+    bfv::adj_reduce_kernel<float><<<nblocks, bfv::kReduceThreads, 0, st>>>(
         static_cast<const float *>(mu), static_cast<const float *>(u), nel, n_sub, stride, n_axis,
         used, partial);
-    bfv::adj_reduce_final_kernel<float><<<1, bfv::kReduceFinalThreads, 0, st>>>(partial, kBlocks, n_sub, -dt / 3.0,
-                                                          -dt / (h_axis * h_axis), dlambda, dD);
+    bfv::adj_reduce_final_kernel<float><<<1, bfv::kReduceFinalThreads, 0, st>>>(
+        partial, nblocks, n_sub, -dt / 3.0, -dt / (h_axis * h_axis), dlambda, dD);
   }
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(BIOFVM_ERR_CUDA, cudaGetErrorString(e));
