@@ -19,7 +19,9 @@ struct PipeShape {
   size_t smem = 0;
 };
 struct PipeKnobs {
-  int chunk = 0, cw = 0;  // asked-for chunk length and columns per tile (0: the planner's)
+  // asked-for chunk length and columns per tile (0: the planner's): the chunk capacity that holds it
+  // or the largest of the axis and width, and the planner's own choice where those do not fit
+  int chunk = 0, cw = 0;
   int ns = 4;             // most ring stages per CTA
 };
 
@@ -148,15 +150,23 @@ inline bool pipe_shape(int axis, int64_t nx, int64_t ny, int64_t nz, int64_t S, 
   for (int cw : {32, 24, 16}) {
     if (knobs.cw && cw != knobs.cw) continue;
     for (int target : {16, 24, 48}) {
-      const int want = knobs.chunk > 0 ? knobs.chunk : target;
-      const int maxm = want <= 8 && cw == 32 ? 8 : want <= 16 ? 16 : want <= 24 ? 24 : 48;
+      int maxm = target;
+      if (knobs.chunk > 0) {
+        maxm = knobs.chunk <= 8 ? 8 : knobs.chunk <= 16 ? 16 : knobs.chunk <= 24 ? 24 : 48;
+        if (cw == 24) maxm = 48;
+        else if (!compiled(cw, maxm)) maxm = maxm == 8 ? 16 : 24;
+      }
       const int cpw = pipe_chunks_per_warp(cw), T = (n + maxm - 1) / maxm;
       if (!compiled(cw, maxm) || (T + cpw - 1) / cpw + extra > pipe_sm_warps(maxm)) continue;
       if (fits(cw, maxm, false)) return true;
       break;
     }
   }
-  if (knobs.chunk > 0 || knobs.cw) return false;
+  if (knobs.chunk > 0 || knobs.cw) {
+    PipeKnobs own;
+    own.ns = knobs.ns;
+    return pipe_shape(axis, nx, ny, nz, S, esz, gp, own, p);
+  }
   for (int cw : {32, 24, 16})
     for (int maxm : {16, 24, 48})
       if (compiled(cw, maxm) && fits(cw, maxm, false)) return true;

@@ -57,3 +57,26 @@ def test_long_fp32_lines_at_odd_substrate_counts(lib, shape):
     assert st == binding.OK
     assert host_api.describe(lib, h).count("pipe") == 3
     lib.biofvm_destroy(h)
+
+
+@pytest.mark.parametrize("cw", [0, 16, 24, 32])
+@pytest.mark.parametrize("chunk", [1, 8, 16, 20, 24, 32, 48, 64, 500])
+def test_a_forced_tile_never_refuses_an_axis(lib, chunk, cw):
+    out = (ctypes.c_int * 3)()
+    for axis in range(3):
+        for n, ns in ((40, 1), (400, 4), (1000, 2), (1100, 5)):
+            dims = [8, 8, 8]
+            dims[axis] = n
+            assert lib.stand_in_pipe_shape(axis, *dims, ns, 4, dims[0] * ns, chunk, cw, out)
+            if n == 40 and cw in (0, 32):  # fits: the capacity that holds the length
+                caps = [8, 16, 24] if axis == 0 else [8, 16, 24, 48]
+                assert out[:2] == [32, next((c for c in caps if c >= chunk), caps[-1])]
+
+
+@pytest.mark.parametrize("chunk", ["32", "48"])
+def test_16_bit_handles_under_a_forced_chunk(lib, chunk, monkeypatch):
+    monkeypatch.setenv("BIOFVM_PIPE_CHUNK", chunk)
+    st, h = host_api.create(lib, 64, 64, 64, 2, "fp16")
+    assert st == binding.OK
+    assert host_api.describe(lib, h) == "x=pipe/cw32/m24 y=pipe/cw32/m48 z=pipe/cw32/m48"
+    lib.biofvm_destroy(h)
