@@ -80,6 +80,7 @@ struct ColPlan {
 // the plain kernels).
 struct PipePlan : PipeShape {
   int use = 0, grid = 0;
+  int shared_grid = 0;  // beside the other environments of a batch (batch_share_sms)
   CUtensorMap map[2]{};  // y/z: [0] the field, [1] the adjoint field
   int have_map[2]{};
 };
@@ -151,7 +152,6 @@ struct biofvm {
   PipeKnobs pipe_knobs;      // pipelined sweeps
   DevBuf scratch;            // FP32 streaming: forward intermediate, field-sized
   int forced = 0;  // chunk lengths fixed by the caller (batched environments)
-  int batched = 0;  // an environment of a batch in per-environment mode
   unsigned generation = 0;  // bumped when kernel arguments change (sources, constants)
   // sources
   int64_t n_entries = 0;
@@ -940,8 +940,9 @@ AxisTab axis_tab(const biofvm *h, int axis) {
 // ---------------------------------------------------------------------------
 // Launch the pipelined sweep of `axis` on `field` (buf selects the y/z tensor map).  The
 // row-padded working copy (`pitched`): the plans ppx over it, rows gpitch elements apart.
+// `shared`: beside the sweeps of a batch's other environments.
 cudaError_t launch_pipe(const biofvm *h, int axis, int flags, cudaStream_t st, void *field,
-                        int buf, bool pitched = false) {
+                        int buf, bool pitched = false, bool shared = false) {
   const PipePlan &p = pitched ? h->ppx[axis] : h->pp[axis];
   const int gp = pitched ? h->gpitch : h->g.nx * h->g.n_sub;
   PipeArgs b{};
@@ -989,11 +990,12 @@ cudaError_t launch_pipe(const biofvm *h, int axis, int flags, cudaStream_t st, v
   // Programmatic serialisation (pipe.cuh) where a sweep is short: 113 x 97 x 121 x 3 with its
   // adjoint 2.9% faster, 250^3 0.8%; 400^3 x 4, whose sweeps are bound by HBM, 2% slower, and in a
   // batch, whose other environments fill the gaps, no faster.
-  b.overlap = !h->batched && (double)h->nel * (double)h->esz <= 96.0e6;
+  b.overlap = !shared && (double)h->nel * (double)h->esz <= 96.0e6;
   const CUtensorMap &map = p.map[axis == 0 ? 0 : buf];
-  if (h->prec == BIOFVM_BF16) return launch_pipe_bf16(map, b, p.maxm, p.grid, p.smem, st);
-  if (h->prec == BIOFVM_FP16) return launch_pipe_fp16(map, b, p.maxm, p.grid, p.smem, st);
-  return launch_pipe_f32(map, b, p.maxm, p.grid, p.smem, st);
+  const int grid = shared ? p.shared_grid : p.grid;
+  if (h->prec == BIOFVM_BF16) return launch_pipe_bf16(map, b, p.maxm, grid, p.smem, st);
+  if (h->prec == BIOFVM_FP16) return launch_pipe_fp16(map, b, p.maxm, grid, p.smem, st);
+  return launch_pipe_f32(map, b, p.maxm, grid, p.smem, st);
 }
 
 bool stream_ok(const biofvm *h, int axis, int flags) {
@@ -1070,9 +1072,11 @@ bool pipe_ok(const biofvm *h, int axis, int flags, int buf) {
   return p.use && (flags & kSolve) && (axis == 0 || p.have_map[buf]);
 }
 
-cudaError_t launch_x(const biofvm *h, int flags, cudaStream_t st, void *field = nullptr) {
+cudaError_t launch_x(const biofvm *h, int flags, cudaStream_t st, void *field = nullptr,
+                     bool shared = false) {
   if (stream_ok(h, 0, flags)) return launch_stream(h, 0, flags, st, field ? field : h->rho.p);
-  if (pipe_ok(h, 0, flags, 0)) return launch_pipe(h, 0, flags, st, field ? field : h->rho.p, 0);
+  if (pipe_ok(h, 0, flags, 0))
+    return launch_pipe(h, 0, flags, st, field ? field : h->rho.p, 0, false, shared);
   if ((flags & kSolve) && h->xp.nosolve) return cudaErrorInvalidConfiguration;
   XLaunch a{};
   a.rho = field ? field : h->rho.p;
@@ -1103,7 +1107,8 @@ cudaError_t launch_x(const biofvm *h, int flags, cudaStream_t st, void *field = 
   return h->prec == BIOFVM_FP64 ? launch_x_f64(a, st) : launch_x_f32(a, st);
 }
 
-cudaError_t launch_col(const biofvm *h, int axis, int flags, cudaStream_t st, int buf = 0) {
+cudaError_t launch_col(const biofvm *h, int axis, int flags, cudaStream_t st, int buf = 0,
+                       bool shared = false) {
   ColLaunch a{};
   a.rho = buf ? h->adj.p : h->rho.p;
   const int64_t nx = h->g.nx, ny = h->g.ny, nz = h->g.nz, S = h->g.n_sub;
@@ -1131,7 +1136,8 @@ cudaError_t launch_col(const biofvm *h, int axis, int flags, cudaStream_t st, in
   a.dir_on = static_cast<const uint8_t *>(h->dir_on_d.p);
   a.dir_val = h->dir_val_d.p;
   if (stream_ok(h, axis, flags)) return launch_stream(h, axis, flags, st, a.rho);
-  if (pipe_ok(h, axis, flags, buf)) return launch_pipe(h, axis, flags, st, a.rho, buf);
+  if (pipe_ok(h, axis, flags, buf))
+    return launch_pipe(h, axis, flags, st, a.rho, buf, false, shared);
   if (h->cp[axis].nosolve) return cudaErrorInvalidConfiguration;
   return h->prec == BIOFVM_FP64 ? launch_col_f64(a, st) : launch_col_f32(a, st);
 }
@@ -1198,23 +1204,24 @@ cudaError_t launch_src(const biofvm *h, cudaStream_t st) {
 bool adjoint_pitched(const biofvm *h) { return h->pitched && !h->any_dir && h->n_dnode == 0; }
 
 // `pitched`: the three pipelined sweeps on the row-padded working copy (no
-// Dirichlet nodes then).
+// Dirichlet nodes then).  `shared`: beside a batch's other environments.
 biofvm_status launch_step(const biofvm *h, cudaStream_t st, int m = 0, bool renorm = true,
-                          bool pitched = false) {
+                          bool pitched = false, bool shared = false) {
   if (pitched) {
-    CK(launch_pipe(h, 0, kSrc | kDirBefore | kSolve | kDirAfter, st, h->prow.p, 0, true));
-    CK(launch_pipe(h, 1, kSolve | kDirAfter, st, h->prow.p, 0, true));
-    CK(launch_pipe(h, 2, kSolve | kDirAfter, st, h->prow.p, 0, true));
+    CK(launch_pipe(h, 0, kSrc | kDirBefore | kSolve | kDirAfter, st, h->prow.p, 0, true, shared));
+    CK(launch_pipe(h, 1, kSolve | kDirAfter, st, h->prow.p, 0, true, shared));
+    CK(launch_pipe(h, 2, kSolve | kDirAfter, st, h->prow.p, 0, true, shared));
     return BIOFVM_OK;
   }
   const int sc = step_scaled(h);
   const int mf = sc ? (m << 8) : 0;
   CK(launch_nodes(h, st, m, sc ? 0 : -1));
-  CK(launch_x(h, kSrc | kDirBefore | kSolve | kDirAfter | sc | mf, st));
+  CK(launch_x(h, kSrc | kDirBefore | kSolve | kDirAfter | sc | mf, st, nullptr, shared));
   CK(launch_nodes(h, st, m, sc ? 6 : -1));
-  CK(launch_col(h, 1, kSolve | kDirAfter | sc | mf, st));
+  CK(launch_col(h, 1, kSolve | kDirAfter | sc | mf, st, 0, shared));
   CK(launch_nodes(h, st, m, sc ? 7 : -1));
-  CK(launch_col(h, 2, kSolve | kDirAfter | sc | mf | (sc && !renorm ? kKeepScale : 0), st));
+  CK(launch_col(h, 2, kSolve | kDirAfter | sc | mf | (sc && !renorm ? kKeepScale : 0), st, 0,
+                shared));
   CK(launch_nodes(h, st, m, sc && !renorm ? 8 : -1));
   return BIOFVM_OK;
 }
@@ -2317,7 +2324,7 @@ biofvm_status batch_capture_graph_mode(biofvm_batch *b, int K) {
   for (int i = 0; i < ne && e == cudaSuccess && st == BIOFVM_OK; i++) {
     const biofvm *h = b->env[i];
     for (int k = 0; k < K && st == BIOFVM_OK; k++)
-      st = launch_step(h, b->fork[b->fork_of[i]], 0, true, h->pitched != 0);
+      st = launch_step(h, b->fork[b->fork_of[i]], 0, true, h->pitched != 0, true);
   }
   for (int f = 0; f < nf && e == cudaSuccess; f++) {
     e = cudaEventRecord(b->fork_ev[1 + f], b->fork[f]);
@@ -2340,8 +2347,8 @@ biofvm_status batch_capture_graph_mode(biofvm_batch *b, int K) {
   return BIOFVM_OK;
 }
 
-// Per-environment mode: the environments' sweeps run side by side, so a sweep need not spread
-// over every SM it can fill.  With many tiles in all, at least four tiles a CTA: its constants
+// Per-environment mode: the environments' sweeps run side by side, so a sweep of the batch's own
+// step need not spread over every SM it can fill (a step of one environment's handle does).  With many tiles in all, at least four tiles a CTA: its constants
 // and the first tile's latency are then paid a quarter as often (20 environments of 64..128
 // voxels: 429 us a step with a CTA per tile where they fit, 365 with two tiles, 317 with four,
 // 335 with eight; two environments, 1014 tiles: 33.2, 32.3, 37.1 and 55.4).
@@ -2355,7 +2362,8 @@ void batch_share_sms(biofvm_batch *b) {
       const int64_t per = std::max<int64_t>(1, std::min<int64_t>(4, total / (8 * h->num_sms)));
       for (PipePlan *p : {&h->pp[axis], &h->ppx[axis]})
         if (p->use)
-          p->grid = (int)std::min<int64_t>(p->grid, std::max<int64_t>(1, p->ntiles / per));
+          p->shared_grid =
+              (int)std::min<int64_t>(p->grid, std::max<int64_t>(1, p->ntiles / per));
     }
   }
 }
@@ -2490,7 +2498,6 @@ biofvm_status biofvm_batch_create(int n_env, const biofvm_grid *grids, const dou
       batch_destroy_impl(b);
       return fail(st, "environment %d: %s", e, msg.c_str());
     }
-    h->batched = b->graph_mode;
     b->env.push_back(h);
     b->env_gen.push_back(0);
     b->whole.push_back({whole[0], whole[1], whole[2]});

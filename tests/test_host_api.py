@@ -80,3 +80,22 @@ def test_16_bit_handles_under_a_forced_chunk(lib, chunk, monkeypatch):
     assert st == binding.OK
     assert host_api.describe(lib, h) == "x=pipe/cw32/m24 y=pipe/cw32/m48 z=pipe/cw32/m48"
     lib.biofvm_destroy(h)
+
+
+@pytest.mark.parametrize("grid", [(96, 96, 96, 2), (97, 95, 96, 1)], ids=["aligned", "padded"])
+def test_a_batch_environments_own_step_takes_the_whole_gpu(lib, grid, monkeypatch):
+    monkeypatch.setenv("BIOFVM_BATCH_MODE", "graph")
+    st, h = host_api.create(lib, *grid, "fp32")
+    st_b, b = host_api.create_batch(lib, [grid] * 12, "fp32")
+    assert st == st_b == binding.OK
+    env = ctypes.c_void_p()
+    assert lib.biofvm_batch_env(b, 3, ctypes.byref(env)) == binding.OK
+    seen = []
+    for step, what in ((lib.biofvm_step, h), (lib.biofvm_step, env), (lib.biofvm_batch_step, b)):
+        lib.stand_in_forget_launches()
+        assert step(what, 1) == binding.OK
+        seen.append([(r.grid, r.overlap) for r in host_api.pipe_launches(lib)[:3]])
+    assert seen[1] == seen[0]
+    assert all(batch[0] < alone[0] and not batch[1] for batch, alone in zip(seen[2], seen[0]))
+    lib.biofvm_destroy(h)
+    lib.biofvm_batch_destroy(b)
