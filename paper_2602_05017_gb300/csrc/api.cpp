@@ -1298,7 +1298,12 @@ biofvm_status build_sources(biofvm *h) {
   const size_t u = elem.size();
   for (int64_t r = 0; r < nrows; r++) off[r + 1] += off[r];
   CK(cudaStreamSynchronize(h->stream));  // the kernels may still read the old lists
+  // Until every new list is on the device there is none, and no graph over buffers that go.
   h->n_entries = 0;
+  h->h_entry.assign((size_t)n * S, -1);
+  h->agents_on_device = false;  // the adjoint's agent-to-entry map follows the list
+  h->generation++;
+  drop_graphs(h);
   if (dev_alloc(h->src_row_off, off.size() * 8) != cudaSuccess)
     return fail(BIOFVM_ERR_OOM, "device allocation for the source offsets failed");
   CK(cudaMemcpy(h->src_row_off.p, off.data(), off.size() * 8, cudaMemcpyHostToDevice));
@@ -1317,9 +1322,6 @@ biofvm_status build_sources(biofvm *h) {
   h->n_entries = (int64_t)u;
   h->h_entry.swap(entry);
   h->sources_device = false;
-  h->agents_on_device = false;  // the adjoint's agent-to-entry map follows the list
-  h->generation++;
-  drop_graphs(h);  // kernel arguments changed
   return BIOFVM_OK;
 }
 
@@ -1740,6 +1742,8 @@ biofvm_status biofvm_set_dirichlet_nodes(biofvm_t *h, int64_t n, const int64_t *
   }
   CK(cudaStreamSynchronize(h->stream));  // launches in flight may read the old lists
   h->n_dnode = 0;
+  h->generation++;
+  drop_graphs(h);  // (they read the old lists, which an allocation below may give back and fail)
   if (!kel.empty()) {
     if (dev_alloc(h->dn_elem, kel.size() * 8) != cudaSuccess)
       return fail(BIOFVM_ERR_OOM, "device allocation for %zu Dirichlet nodes failed", kel.size());

@@ -99,3 +99,38 @@ def test_a_batch_environments_own_step_takes_the_whole_gpu(lib, grid, monkeypatc
     assert all(batch[0] < alone[0] and not batch[1] for batch, alone in zip(seen[2], seen[0]))
     lib.biofvm_destroy(h)
     lib.biofvm_batch_destroy(b)
+
+
+def test_a_failed_upload_leaves_no_sources_and_a_matching_map(lib):
+    nvox, ns = 16 * 12 * 10, 2
+    st, h = host_api.create(lib, 16, 12, 10, ns, "fp32")
+    assert st == binding.OK
+
+    def agents(n):
+        rates = np.ones((n, ns))
+        voxel = np.arange(n, dtype=np.int64) % nvox
+        return lib.biofvm_set_sources(h, n, *(ctypes.c_void_p(a.ctypes.data) for a in (
+            voxel, rates, rates, rates)), None)
+
+    def adjoint():  # entries walked, entries of the map, largest entry, entries of the list
+        field, saved = np.zeros(nvox * ns, np.float32), np.zeros(4 * nvox * ns, np.float32)
+        grads = [np.zeros(4096) for _ in range(3)]
+        ptr = [ctypes.c_void_p(a.ctypes.data) for a in (field, field, *grads, saved)]
+        assert lib.biofvm_adjoint_step(h, *ptr) == binding.OK
+        out = (ctypes.c_int64 * 4)()
+        lib.stand_in_source_adjoint(out)
+        return list(out)
+
+    for n in (5, 700, 3):
+        assert agents(n) == binding.OK
+        assert adjoint() == [n * ns, adjoint()[1], n * ns - 1, n * ns] and adjoint()[1] >= n * ns
+        graphs = lib.stand_in_graphs_made()
+        assert lib.biofvm_step(h, 1) == binding.OK
+        lib.stand_in_fail_allocation(0)
+        assert agents(1500) == binding.ERR_OOM
+        lib.stand_in_fail_allocation(-1)
+        walked, held, largest, entries = adjoint()
+        assert walked == 1500 * ns and held >= walked and largest == -1 and entries == 0
+        assert lib.biofvm_step(h, 1) == binding.OK  # a new graph: the old one reads freed lists
+        assert lib.stand_in_graphs_made() == graphs + 2
+    lib.biofvm_destroy(h)
