@@ -163,7 +163,8 @@ struct biofvm {
   bool sources_device = false;
   DevBuf dsrc_row_off, dsrc_elem, dsrc_rowcol, dsrc_alpha, dsrc_scale, dsrc_count;
   DevBuf ag_key[2], ag_idx[2], ag_ea, ag_eb, ag_head, ag_pos, ag_hist, ag_part, ag_count32;
-  // step graphs: [0] a block of renorm_k steps, [r] a tail of r < renorm_k steps
+  // step graphs: [0] a block of renorm_k steps, [r] a tail of r < renorm_k steps ([1] on the
+  // row-padded copy, where renorm_k is 1: a step with its copies)
   cudaGraph_t graph[kMaxRenorm + 1] = {};
   cudaGraphExec_t gexec[kMaxRenorm + 1] = {};
   // FP64 streaming step: the field stays scaled by omega^-m for m < renorm_k
@@ -1961,22 +1962,23 @@ biofvm_status biofvm_step(biofvm_t *h, int n_steps) {
   // graphs are dropped whenever nodes are set, so they never mix the two forms)
   const int K = step_scaled(h) ? h->renorm_k : 1;
   const bool pitched = h->pitched && h->n_dnode == 0;
-  // slot 0: K steps; slot r: r < K steps.  Pitched (K = 1): slots 2, 3 and 4 are a step with the
-  // copy in before it, the copy out after it, and both.
+  // slot 0: K steps; slot r: r < K steps.  Pitched (K = 1): slot 1 is a step with its copies, the
+  // whole of a one-step call (41 x 37 x 29 x 2: 28.8 us, 34.8 with the copies launched beside the
+  // graph); a longer call launches its copies, and so never makes a second graph.
   auto ensure = [&](int slot) -> biofvm_status {
     if (h->gexec[slot]) return BIOFVM_OK;
-    const int r = slot == 0 ? K : pitched ? 1 : slot;
-    const bool in = pitched && (slot == 2 || slot == 4), out = pitched && slot >= 3;
+    const int r = slot == 0 ? K : slot;
+    const bool copies = pitched && slot == 1;
     CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
     biofvm_status st = BIOFVM_OK;
     auto copy = [&](bool way) -> biofvm_status {
       CK(pitch_copy(h, way, h->cap_stream));
       return BIOFVM_OK;
     };
-    if (in) st = copy(true);
+    if (copies) st = copy(true);
     for (int m = 0; m < r && st == BIOFVM_OK; m++)
       st = launch_step(h, h->cap_stream, m, m == r - 1, pitched);
-    if (out && st == BIOFVM_OK) st = copy(false);
+    if (copies && st == BIOFVM_OK) st = copy(false);
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamEndCapture(h->cap_stream, &graph);
     if (st != BIOFVM_OK) {
@@ -1993,17 +1995,15 @@ biofvm_status biofvm_step(biofvm_t *h, int n_steps) {
     h->graph[slot] = graph;
     return BIOFVM_OK;
   };
-  // the call's graphs: `first` once, slot 0 `mid` times, `last` once (-1: none)
-  const int tail = n_steps % K;
-  const int first = !pitched ? -1 : n_steps == 1 ? 4 : 2;
-  const int last = pitched ? (n_steps == 1 ? -1 : 3) : tail > 0 ? tail : -1;
-  const int mid = pitched ? std::max(0, n_steps - 2) : n_steps / K;
+  const bool one = pitched && n_steps == 1;
+  const int blocks = one ? 0 : n_steps / K, tail = one ? 1 : n_steps % K;
   biofvm_status st;  // every graph before anything is launched
-  for (int slot : {first, mid > 0 ? 0 : -1, last})
-    if (slot >= 0 && (st = ensure(slot)) != BIOFVM_OK) return st;
-  if (first >= 0) CK(cudaGraphLaunch(h->gexec[first], h->stream));
-  for (int b = 0; b < mid; b++) CK(cudaGraphLaunch(h->gexec[0], h->stream));
-  if (last >= 0) CK(cudaGraphLaunch(h->gexec[last], h->stream));
+  if (blocks > 0 && (st = ensure(0)) != BIOFVM_OK) return st;
+  if (tail > 0 && (st = ensure(tail)) != BIOFVM_OK) return st;
+  if (pitched && !one) CK(pitch_copy(h, true, h->stream));
+  for (int b = 0; b < blocks; b++) CK(cudaGraphLaunch(h->gexec[0], h->stream));
+  if (tail > 0) CK(cudaGraphLaunch(h->gexec[tail], h->stream));
+  if (pitched && !one) CK(pitch_copy(h, false, h->stream));
   return BIOFVM_OK;
 }
 

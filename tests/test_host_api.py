@@ -134,3 +134,15 @@ def test_a_failed_upload_leaves_no_sources_and_a_matching_map(lib):
         assert lib.biofvm_step(h, 1) == binding.OK  # a new graph: the old one reads freed lists
         assert lib.stand_in_graphs_made() == graphs + 2
     lib.biofvm_destroy(h)
+
+
+@pytest.mark.parametrize("steps", [1, 2, 3, 10])
+@pytest.mark.parametrize("grid", [(41, 37, 29, 2), (64, 32, 16, 2)], ids=["padded", "aligned"])
+def test_one_graph_a_call(lib, grid, steps):
+    st, h = host_api.create(lib, *grid, "fp32")
+    assert st == binding.OK
+    graphs = lib.stand_in_graphs_made()
+    for _ in range(3):
+        assert lib.biofvm_step(h, steps) == binding.OK
+    assert lib.stand_in_graphs_made() == graphs + 1
+    lib.biofvm_destroy(h)
