@@ -125,9 +125,9 @@ struct biofvm {
   // FP32 fields whose rows (nx*S elements) are not 16-byte multiples, which the TMA copies
   // need: biofvm_step runs the pipelined sweeps on a row-padded working copy (rows gpitch
   // elements apart, the padding zero), copied in at the start of the call and back at its
-  // end.  ppx: the plans over that copy; tabP / tabTP: the axis tables of their partitions
+  // end.  ppx: the plans over that copy; tabTP: their constants
   int pitched = 0, gpitch = 0, pitched_enabled = 1;
-  DevBuf prow, tabP[3], tabTP[3];
+  DevBuf prow, tabTP[3];
   PipePlan ppx[3];
   StreamPlan sp[3];
   int num_sms = 0;
@@ -806,13 +806,11 @@ biofvm_status upload_constants(biofvm *h) {
       else line_tables(h, axis, h->small_T[axis], h->small_m[axis], f32, ts);
       if ((st = upload_doubles(h, h->small_tab[axis], ts)) != BIOFVM_OK) return st;
     }
-    // the row-padded working copy's plans: tables of their own partition
+    // the row-padded working copy's plans: constants of their own partition
     const PipePlan &q = h->ppx[axis];
     if (h->pitched) {
       axis_tables(h, axis, q.T, q.m, f32, t);
-      if ((st = upload_doubles(h, h->tabP[axis], t)) != BIOFVM_OK ||
-          (st = upload_T(h->tabTP[axis], q)) != BIOFVM_OK)
-        return st;
+      if ((st = upload_T(h->tabTP[axis], q)) != BIOFVM_OK) return st;
     }
   }
   if (h->prec != BIOFVM_FP64) {
@@ -909,11 +907,12 @@ SrcLists src_lists(const biofvm *h) {
   return l;
 }
 
-// The tables of an axis (layout of axis_tables, chunk partition T x m) as kernel arguments.
-AxisTab axis_tab_of(const biofvm *h, int axis, const DevBuf &tab, const DevBuf &tabT, int T,
-                    int m) {
+// The tables of an axis (layout of axis_tables) as kernel arguments.
+AxisTab axis_tab(const biofvm *h, int axis) {
+  int T, m;
+  axis_partition(h, axis, T, m);
   const int n = axis_len(h, axis), S = h->g.n_sub;
-  const char *base = static_cast<const char *>(tab.p);
+  const char *base = static_cast<const char *>(h->tab[axis].p);
   const size_t blk = (size_t)n * S * h->csz;
   AxisTab t;
   t.inv = base;
@@ -923,17 +922,11 @@ AxisTab axis_tab_of(const biofvm *h, int axis, const DevBuf &tab, const DevBuf &
   t.pc = base + 4 * blk;
   t.cfix = base + 4 * blk + (size_t)T * S * h->csz;
   t.cw = base + 4 * blk + ((size_t)T * S + 2 * (size_t)S) * h->csz;
-  t.tabT = tabT.p;
+  t.tabT = h->tabT[axis].p;
   t.n = n;
   t.T = T;
   t.m = m;
   return t;
-}
-
-AxisTab axis_tab(const biofvm *h, int axis) {
-  int T, m;
-  axis_partition(h, axis, T, m);
-  return axis_tab_of(h, axis, h->tab[axis], h->tabT[axis], T, m);
 }
 
 // ---------------------------------------------------------------------------
@@ -969,11 +962,8 @@ cudaError_t launch_pipe(const biofvm *h, int axis, int flags, cudaStream_t st, v
   b.field = field;
   b.stages = p.stages;
   b.stage_elems = p.stage_elems;
-  b.tab = pitched
-              ? axis_tab_of(h, axis, h->tabP[axis], h->tabTP[axis], p.T, p.m)
-              : axis_tab(h, axis);
+  b.tab.tabT = pitched ? h->tabTP[axis].p : h->tabT[axis].p;  // (the pipeline reads no other table)
   b.tab.T = p.T;
-  b.tab.m = p.m;
   b.k0 = h->stream_k0[axis];
   b.flags = flags;
   if (!h->any_dir) b.flags &= ~(kDirBefore | kDirAfter);
@@ -1363,8 +1353,7 @@ void destroy_impl(biofvm *h) {
                     &h->ag_key[0], &h->ag_key[1], &h->ag_idx[0], &h->ag_idx[1], &h->ag_ea,
                     &h->ag_eb, &h->ag_head, &h->ag_pos, &h->ag_hist, &h->ag_part,
                     &h->ag_count32, &h->small_bar, &h->small_tab[0], &h->small_tab[1],
-                    &h->small_tab[2], &h->prow, &h->tabP[0], &h->tabP[1],
-                    &h->tabP[2], &h->tabTP[0], &h->tabTP[1], &h->tabTP[2]})
+                    &h->small_tab[2], &h->prow, &h->tabTP[0], &h->tabTP[1], &h->tabTP[2]})
     b->release();
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   delete h;
