@@ -276,21 +276,19 @@ void axis_tables(const biofvm *h, int axis, int T, int m, bool defect, std::vect
 }
 
 // Tables of the warp-level line solves (LineTab) of one axis, T chunks of m positions:
-// inv, mul [T*m][S], scan weights [log2 T][2][T][S], c_hi, c_lo [2][S].
-void line_tables(const biofvm *h, int axis, int T, int m, bool defect, std::vector<double> &out) {
+// inv, mul [T*m][S], scan weights [log2 T][2][T][S].
+void line_tables(const biofvm *h, int axis, int T, int m, std::vector<double> &out) {
   const int n = axis_len(h, axis), S = h->g.n_sub, np = T * m;
   std::vector<double> t;
-  axis_tables(h, axis, (n + m - 1) / m, m, defect, t);
+  axis_tables(h, axis, (n + m - 1) / m, m, false, t);
   const int Tn = (n + m - 1) / m;  // chunks that hold positions
-  const double *inv = t.data(), *mul = inv + (size_t)n * S, *pc = mul + 3 * (size_t)n * S,
-               *cfix = pc + (size_t)Tn * S;
+  const double *inv = t.data(), *mul = inv + (size_t)n * S, *pc = mul + 3 * (size_t)n * S;
   int lg = 0;
   while ((1 << lg) < T) lg++;
-  out.assign((size_t)2 * np * S + (size_t)2 * lg * T * S + 2 * (size_t)S, 0.0);
-  double *wt = out.data() + (size_t)2 * np * S, *cf = wt + (size_t)2 * lg * T * S;
+  out.assign((size_t)2 * np * S + (size_t)2 * lg * T * S, 0.0);
+  double *wt = out.data() + (size_t)2 * np * S;
   std::copy(inv, inv + (size_t)n * S, out.begin());
   std::copy(mul, mul + (size_t)n * S, out.begin() + (size_t)np * S);
-  std::copy(cfix, cfix + 2 * (size_t)S, cf);
   auto prod = [&](int lo, int hi, int s) {  // over whole chunks lo..hi
     double x = 1.0;
     for (int u = std::max(lo, 0); u <= hi; u++) x *= u < Tn ? pc[(size_t)u * S + s] : 0.0;
@@ -306,14 +304,11 @@ void line_tables(const biofvm *h, int axis, int T, int m, bool defect, std::vect
 
 LineTab line_tab(const biofvm *h, int axis, int T, int m, const DevBuf &b) {
   const int S = h->g.n_sub, np = T * m;
-  int lg = 0;
-  while ((1 << lg) < T) lg++;
   const char *base = static_cast<const char *>(b.p);
   LineTab t;
   t.inv = base;
   t.mul = base + (size_t)np * S * h->csz;
   t.wt = base + (size_t)2 * np * S * h->csz;
-  t.cfix = base + ((size_t)2 * np * S + (size_t)2 * lg * T * S) * h->csz;
   t.n = axis_len(h, axis);
   t.T = T;
   t.m = m;
@@ -803,7 +798,7 @@ biofvm_status upload_constants(biofvm *h) {
     if (h->small_use) {
       std::vector<double> ts;
       if (h->small_planes) axis_tables(h, axis, h->small_T[axis], h->small_m[axis], false, ts);
-      else line_tables(h, axis, h->small_T[axis], h->small_m[axis], f32, ts);
+      else line_tables(h, axis, h->small_T[axis], h->small_m[axis], ts);
       if ((st = upload_doubles(h, h->small_tab[axis], ts)) != BIOFVM_OK) return st;
     }
     // the row-padded working copy's plans: constants of their own partition

@@ -221,8 +221,8 @@ constexpr int small_warps(int maxm) { return maxm <= 8 ? 16 : 12; }
 cudaError_t launch_small_f64(const SmallArgs &a, int maxm, int grid, int threads, bool cluster,
                              cudaStream_t st);
 // The same for grids with lines of more than 128 voxels (small_planes.cu).
-// Planes of nx*ny*S elements in shared memory for the x and y solves, z-lines
-// by the streaming line solver; bar: 3 words (arrivals, generation, abort) of
+// Planes of nx*ny*S elements, then groups of 32 z-lines, solved in shared
+// memory; bar: 3 words (arrivals, generation, abort) of
 // the bounded grid barrier, zeroed before each launch.
 struct PlanesArgs {
   double *rho;

@@ -8,9 +8,8 @@
 // another's latency.  Lanes without a line, and positions past a line's end,
 // have zero values and zero coefficients.
 //
-// The recurrences (App. A; FP32 in defect-correction form, AxisTab) run twice
-// in either direction: from a zero carry for the chunk's end value, then from
-// the true carry.  The end values meet in a Kogge-Stone scan over the chunks,
+// The recurrences (App. A) run twice in either direction: from a zero carry for
+// the chunk's end value, then from the true carry.  The end values meet in a Kogge-Stone scan over the chunks,
 // weighted with products of mul that the host forms in FP64.
 //
 // The field is read through L1, where the lanes of neighbouring items (a CTA
@@ -21,7 +20,6 @@
 #include <stdint.h>
 
 #include "lines_args.h"
-#include "sweeps.cuh"
 
 namespace bfv {
 
@@ -46,7 +44,6 @@ __device__ __forceinline__ void solve_item(E *p, long long ps, int len, int lo, 
   const unsigned FULL = 0xffffffffu;
   const int n = tb.n, T = tb.T, m = tb.m, lpw = 32 / T, t = lane / lpw;
   E v[MAXM], mu[MAXM];
-  E d[kDefect<E> ? MAXM : 1];
 #pragma unroll
   for (int i = 0; i < MAXM; i++) v[i] = i < len ? p[i * ps] : E(0);
   const E *const t_inv = static_cast<const E *>(tb.inv) + (size_t)lo * S + s;
@@ -58,24 +55,6 @@ __device__ __forceinline__ void solve_item(E *p, long long ps, int len, int lo, 
 #pragma unroll
     for (int i = 0; i < MAXM; i++)
       if (i < len && before.at(lo + i, n)) v[i] = before.val;
-  }
-  if constexpr (kDefect<E>) {
-    // e = L_N d with mirrored ends (d_{-1} = d_0, d_n = d_{n-1})
-    E last = v[0];
-#pragma unroll
-    for (int i = 1; i < MAXM; i++)
-      if (i < m) last = v[i];
-    E left = __shfl_up_sync(FULL, last, lpw), right = __shfl_down_sync(FULL, v[0], lpw);
-    if (t == 0) left = v[0];
-    E am = left - v[0];
-#pragma unroll
-    for (int i = 0; i < MAXM; i++) {
-      d[i] = v[i];
-      const E nxt = lo + i >= n - 1 ? v[i] : (i + 1 < MAXM && i + 1 < m) ? v[i + 1 < MAXM ? i + 1 : i] : right;
-      const E a = v[i] - nxt;
-      v[i] = a - am;  // (d_i - d_{i-1}) + (d_i - d_{i+1})
-      am = a;
-    }
   }
   E g = E(0);
 #pragma unroll
@@ -114,12 +93,6 @@ __device__ __forceinline__ void solve_item(E *p, long long ps, int len, int lo, 
       x = fma(mu[i], x, v[i]);
       v[i] = x;
     }
-  if constexpr (kDefect<E>) {  // x = c_hi d + (c_lo d + y), one final rounding
-    const E chi = __ldg(static_cast<const E *>(tb.cfix) + s);
-    const E clo = __ldg(static_cast<const E *>(tb.cfix) + S + s);
-#pragma unroll
-    for (int i = 0; i < MAXM; i++) v[i] = fma(chi, d[i], fma(clo, d[i], v[i]));
-  }
   if (__any_sync(FULL, after.on)) {
 #pragma unroll
     for (int i = 0; i < MAXM; i++)

@@ -8,7 +8,6 @@ struct LineTab {
   const void *inv, *mul;  // [T * m][S] of every position (0 past the line)
   const void *wt;         // [log2 T][2][T][S] scan weights: forward, the product of mul over
                           // chunks t - 2^k + 1 .. t; backward, over t .. t + 2^k - 1
-  const void *cfix;       // FP32: c_hi, c_lo [2][S]
   int n, T, m;            // T chunks (a power of two) of m positions
 };
 

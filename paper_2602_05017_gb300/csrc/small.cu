@@ -26,6 +26,7 @@
 
 #include <algorithm>
 
+#include "internal.h"
 #include "lines.cuh"
 
 namespace bfv {
