@@ -20,7 +20,7 @@ SOURCES = ["api.cpp", "sweeps_fp64.cu", "sweeps_fp32.cu", "pipe_fp32.cu", "pipe_
            "probe.cu", "agents.cu", "small.cu",
            "small_planes.cu"]
 HEADERS = ["internal.h", "sweeps.cuh", "pipe.cuh", "pipe_args.h", "pipe_plan.h", "adjoint.cuh", "batch.cuh", "batch_args.h",
-           "stream.cuh", "agents.h", "lines.cuh", "lines_args.h"]
+           "stream.cuh", "agents.h", "grid_sync.cuh", "lines.cuh", "lines_args.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -582,7 +582,7 @@ void plan_small(biofvm *h) {
     cudaGetLastError();
     return;
   }
-  if (dev_alloc(h->small_bar, 16) != cudaSuccess) {
+  if (dev_alloc(h->small_bar, 8) != cudaSuccess) {
     cudaGetLastError();
     return;
   }
@@ -1927,7 +1927,7 @@ biofvm_status biofvm_step(biofvm_t *h, int n_steps) {
         a.T[axis] = h->small_T[axis];
         a.m[axis] = h->small_m[axis];
       }
-      CK(cudaMemsetAsync(h->small_bar.p, 0, 16, h->stream));
+      CK(cudaMemsetAsync(h->small_bar.p, 0, 8, h->stream));
       CK(launch_planes_f64(a, h->small_grid, h->small_smem, h->stream));
       return BIOFVM_OK;
     }

@@ -222,8 +222,7 @@ cudaError_t launch_small_f64(const SmallArgs &a, int maxm, int grid, int threads
                              cudaStream_t st);
 // The same for grids with lines of more than 128 voxels (small_planes.cu).
 // Planes of nx*ny*S elements, then groups of 32 z-lines, solved in shared
-// memory; bar: 3 words (arrivals, generation, abort) of
-// the bounded grid barrier, zeroed before each launch.
+// memory; bar as above.
 struct PlanesArgs {
   double *rho;
   int nx, ny, nz, S;

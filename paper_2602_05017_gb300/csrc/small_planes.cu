@@ -25,17 +25,13 @@
 //     the way back to the field;
 //   grid barrier, next step.
 //
-// The grid barrier is a counter and a generation word in global memory; every
-// wait on it is bounded (about two seconds): on expiry the status word is set,
-// an abort word makes every CTA stop at its next barrier, and the launch
-// returns (the field is then undefined).  All CTAs are co-resident: the
-// launch goes through cudaLaunchCooperativeKernel, which refuses a grid that
-// could not be.
+// The barrier is grid_sync.cuh's.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include <algorithm>
 
+#include "grid_sync.cuh"
 #include "internal.h"
 
 namespace bfv {
@@ -43,50 +39,6 @@ namespace bfv {
 namespace {
 
 constexpr int kPlanesThreads = 256;
-
-__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
-// Barrier of all CTAs; false when it gave up (timeout, or another CTA's).
-// bar[0] arrivals, bar[1] generation, bar[2] abort.
-__device__ bool grid_barrier(unsigned *bar, int *status) {
-  __shared__ int s_ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int ok = ld_acquire_u32(bar + 2) == 0;
-    if (ok) {
-      const unsigned gen = ld_acquire_u32(bar + 1);
-      __threadfence();  // this block's writes (ordered by __syncthreads) before the arrival
-      if (atomicAdd(bar, 1u) + 1 == gridDim.x) {
-        atomicExch(bar, 0u);
-        __threadfence();
-        atomicAdd(bar + 1, 1u);  // release the others
-      } else {
-        const long long t0 = clock64();
-        while (ld_acquire_u32(bar + 1) == gen) {
-          if (ld_acquire_u32(bar + 2) != 0) {
-            ok = 0;
-            break;
-          }
-          if (clock64() - t0 > (1ll << 32)) {
-            atomicExch(status, kStatusTimeout);
-            atomicExch(bar + 2, 1u);
-            ok = 0;
-            break;
-          }
-          __nanosleep(32);
-        }
-      }
-      __threadfence();
-    }
-    s_ok = ok;
-  }
-  __syncthreads();
-  return s_ok != 0;
-}
 
 // One axis's tables staged in shared memory: inv, mul, pf, pb [n][S] (the
 // layout of the host's axis tables) and the carry weights cw [T][T][S].
@@ -190,6 +142,7 @@ __global__ void __launch_bounds__(kPlanesThreads, 1) planes_steps_kernel(const P
     __syncthreads();
   };
   const int ngroups = (pl + 31) / 32;
+  unsigned want = 0;
   for (int step = 0; step < a.n_steps; step++) {
     // ---- phase 1: Src, B, X^-1, B, Y^-1, B on each z-plane in shared memory ----
     for (int z = blockIdx.x; z < nz; z += gridDim.x) {
@@ -218,7 +171,7 @@ __global__ void __launch_bounds__(kPlanesThreads, 1) planes_steps_kernel(const P
       for (int e = threadIdx.x; e < pl; e += blockDim.x) g[e] = buf[e];
       __syncthreads();
     }
-    if (!grid_barrier(a.bar, a.status)) return;
+    if (!grid_barrier<false>(a.bar, want += gridDim.x, a.status)) return;
     // ---- phase 2: Z^-1 then B on groups of 32 adjacent z-lines staged as [z][32] ----
     for (int gi = blockIdx.x; gi < ngroups; gi += gridDim.x) {
       const int c0 = gi * 32, ncol = min(32, pl - c0);
@@ -240,7 +193,7 @@ __global__ void __launch_bounds__(kPlanesThreads, 1) planes_steps_kernel(const P
       }
       __syncthreads();
     }
-    if (!grid_barrier(a.bar, a.status)) return;
+    if (step + 1 < a.n_steps && !grid_barrier<false>(a.bar, want += gridDim.x, a.status)) return;
   }
 }
 
