@@ -52,8 +52,15 @@ __device__ __forceinline__ void small_phase(const SmallArgs &a) {
         const int r0 = it * lpw / a.S, r1 = min(a.ny * a.nz, (it * lpw + lpw - 1) / a.S + 1);
         const long long e0 = __ldg(a.src_row_off + r0), e1 = __ldg(a.src_row_off + r1);
         const long long row_first = (long long)r0 * a.nx * a.S;
-        item_sources<double, MAXM>(v, e0, e1, row_first, (int)(first - row_first), L.len, a.S,
-                                   lane, a.src_elem, a.src_alpha, a.src_scale);
+        if (e1 - e0 <= kFewSources) {
+          item_sources<double, MAXM>(v, e0, e1, row_first, (int)(first - row_first), L.len, a.S,
+                                     lane, a.src_elem, a.src_alpha, a.src_scale);
+        } else {
+          item_sources_in_field<double>(a.rho, e0, e1, row_first, a.nx * a.S, r0, it * lpw, lpw,
+                                        a.S, lane, a.src_elem, a.src_alpha, a.src_scale);
+#pragma unroll
+          for (int i = 0; i < MAXM; i++) v[i] = i < L.len ? a.rho[first + i * L.ps] : 0.0;
+        }
       }
     };
     solve_item<double, MAXM>(a.rho + first, L.ps, L.len, L.lo, L.s, lane, tb, a.S,
