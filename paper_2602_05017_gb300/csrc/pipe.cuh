@@ -489,7 +489,7 @@ __device__ __forceinline__ bool pipe_chunk(const Cols col, const int len, const 
 // MODE 1: y/z tiles (tensor boxes).  PSX > 0 (x tiles only): the substrate
 // count S, known at compile time, so the staged positions (S apart) need no
 // per-access address arithmetic; 0: S read at run time.  CW: columns per tile
-// (32, or 16 for long lines).  H: the field's storage type (E, or bf16 / fp16
+// (32, or 24 or 16 for long lines).  SPLIT: coefficients staged per substrate.  H: the field's storage type (E, or bf16 / fp16
 // with E = float): stages and TMA copies hold H, registers and constants E.
 template <int MAXM, int MODE, int PSX = 0, int CW = 32, typename H = float, bool SPLIT = false>
 __global__ void __maxnreg__(pipe_regs(MAXM))
@@ -882,9 +882,9 @@ __global__ void __maxnreg__(pipe_regs(MAXM))
   }
 }
 
-// Chunk capacities: 8, 16 and 24 positions of 32-column tiles, 16 and 24
-// of 16-column ones; y/z tiles of 32 and 24 columns also 48 (lines whose
-// shorter chunks would take more warps than fit).  x tiles know the substrate count at compile time where it
+// Chunk capacities: 16 and 24 positions of 32- and 16-column tiles; y/z tiles
+// of 32 and 24 columns also 48 (lines whose shorter chunks would take more warps
+// than fit).  x tiles know the substrate count at compile time where it
 // is 1, 2, 4 or 8 (their chunk starts must then be multiples of the positions
 // one access reads: the capacity, or 0).
 template <int MAXM, int CW, typename H, typename F>
@@ -906,8 +906,8 @@ cudaError_t pipe_split_kernels(F &&f) {
   return e != cudaSuccess ? e
                           : f((const void *)sweep_pipe_kernel<kSplitMaxm, 0, 0, CW, H, true>, 0);
 }
-// The second tile width of a capacity (0: none).
-constexpr int pipe_narrow(int maxm) { return maxm <= 8 ? 0 : maxm <= 24 ? 16 : 24; }
+// The second tile width of a capacity.
+constexpr int pipe_narrow(int maxm) { return maxm <= 24 ? 16 : 24; }
 
 template <int MAXM, typename H>
 cudaError_t allow_pipe_smem(size_t bytes) {
@@ -915,8 +915,7 @@ cudaError_t allow_pipe_smem(size_t bytes) {
     return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   };
   cudaError_t e = pipe_kernels<MAXM, 32, H>(set);
-  if constexpr (pipe_narrow(MAXM) > 0)
-    if (e == cudaSuccess) e = pipe_kernels<MAXM, pipe_narrow(MAXM), H>(set);
+  if (e == cudaSuccess) e = pipe_kernels<MAXM, pipe_narrow(MAXM), H>(set);
   if constexpr (MAXM == kSplitMaxm) {
     if (e == cudaSuccess) e = pipe_split_kernels<32, H>(set);
     if (e == cudaSuccess) e = pipe_split_kernels<16, H>(set);
@@ -963,9 +962,8 @@ template <int MAXM, typename H>
 cudaError_t launch_pipe_one(const CUtensorMap &map, const PipeArgs &a, int grid, size_t smem,
                             cudaStream_t st) {
   if (a.cw == 32) return launch_pipe_cw<MAXM, 32, H>(map, a, grid, smem, st);
-  if constexpr (pipe_narrow(MAXM) > 0)
-    if (a.cw == pipe_narrow(MAXM))
-      return launch_pipe_cw<MAXM, pipe_narrow(MAXM), H>(map, a, grid, smem, st);
+  if (a.cw == pipe_narrow(MAXM))
+    return launch_pipe_cw<MAXM, pipe_narrow(MAXM), H>(map, a, grid, smem, st);
   return cudaErrorInvalidConfiguration;
 }
 

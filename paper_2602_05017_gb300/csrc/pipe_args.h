@@ -61,10 +61,10 @@ BFV_HD constexpr int pipe_tab_pairs(int maxm, int S, int W, int chunks_per_warp,
 // counts whose pairs repeat every coefficient.
 constexpr int kSplitMaxm = 24;
 BFV_HD constexpr bool pipe_can_split(int64_t S) { return S > 1 && S % 2 == 1; }
-// Registers of a thread of chunk capacity maxm (the chunk pair takes 2 maxm): 80, 96, 128 and 168
+// Registers of a thread of chunk capacity maxm (the chunk pair takes 2 maxm): 96, 128 and 168
 // hold the solve with few or no spills, and the warps an SM then has room for (its four register files
 // take whole warps) -- also the largest CTA.
-BFV_HD constexpr int pipe_regs(int maxm) { return maxm <= 8 ? 80 : maxm <= 16 ? 96 : maxm <= 24 ? 128 : 168; }
+BFV_HD constexpr int pipe_regs(int maxm) { return maxm <= 16 ? 96 : maxm <= 24 ? 128 : 168; }
 BFV_HD constexpr int pipe_sm_warps(int maxm) { return 4 * (16384 / (pipe_regs(maxm) * 32)); }
 
 struct PipeArgs {

@@ -7,7 +7,6 @@ namespace bfv {
 
 cudaError_t allow_pipe_smem_f32(int maxm, size_t bytes) {
   switch (maxm) {
-    case 8: return allow_pipe_smem<8, float>(bytes);
     case 16: return allow_pipe_smem<16, float>(bytes);
     case 24: return allow_pipe_smem<24, float>(bytes);
     case 48: return allow_pipe_smem<48, float>(bytes);
@@ -18,7 +17,6 @@ cudaError_t allow_pipe_smem_f32(int maxm, size_t bytes) {
 cudaError_t launch_pipe_f32(const CUtensorMap &map, const PipeArgs &a, int maxm, int grid,
                             size_t smem, cudaStream_t st) {
   switch (maxm) {
-    case 8: return launch_pipe_one<8, float>(map, a, grid, smem, st);
     case 16: return launch_pipe_one<16, float>(map, a, grid, smem, st);
     case 24: return launch_pipe_one<24, float>(map, a, grid, smem, st);
     case 48: return launch_pipe_one<48, float>(map, a, grid, smem, st);

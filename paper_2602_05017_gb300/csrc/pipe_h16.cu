@@ -7,7 +7,6 @@ namespace bfv {
 template <typename H>
 cudaError_t allow_pipe_smem_h16(int maxm, size_t bytes) {
   switch (maxm) {
-    case 8: return allow_pipe_smem<8, H>(bytes);
     case 16: return allow_pipe_smem<16, H>(bytes);
     case 24: return allow_pipe_smem<24, H>(bytes);
     case 48: return allow_pipe_smem<48, H>(bytes);
@@ -19,7 +18,6 @@ template <typename H>
 cudaError_t launch_pipe_h16(const CUtensorMap &map, const PipeArgs &a, int maxm, int grid,
                             size_t smem, cudaStream_t st) {
   switch (maxm) {
-    case 8: return launch_pipe_one<8, H>(map, a, grid, smem, st);
     case 16: return launch_pipe_one<16, H>(map, a, grid, smem, st);
     case 24: return launch_pipe_one<24, H>(map, a, grid, smem, st);
     case 48: return launch_pipe_one<48, H>(map, a, grid, smem, st);

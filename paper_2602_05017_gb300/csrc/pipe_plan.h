@@ -141,7 +141,7 @@ inline bool pipe_shape_of(int axis, int64_t nx, int64_t ny, int64_t nz, int64_t 
 inline bool pipe_shape(int axis, int64_t nx, int64_t ny, int64_t nz, int64_t S, size_t esz,
                        int64_t gp, const PipeKnobs &knobs, PipeShape &p) {
   auto compiled = [&](int cw, int maxm) {
-    return maxm == 48 ? axis != 0 && cw != 16 : maxm == 8 ? cw == 32 : cw != 24;
+    return maxm == 48 ? axis != 0 && cw != 16 : cw != 24;
   };
   auto fits = [&](int cw, int maxm, bool split) {
     return pipe_shape_of(axis, nx, ny, nz, S, esz, gp, knobs.ns, cw, maxm, split, p);
@@ -152,9 +152,8 @@ inline bool pipe_shape(int axis, int64_t nx, int64_t ny, int64_t nz, int64_t S, 
     for (int target : {16, 24, 48}) {
       int maxm = target;
       if (knobs.chunk > 0) {
-        maxm = knobs.chunk <= 8 ? 8 : knobs.chunk <= 16 ? 16 : knobs.chunk <= 24 ? 24 : 48;
-        if (cw == 24) maxm = 48;
-        else if (!compiled(cw, maxm)) maxm = maxm == 8 ? 16 : 24;
+        maxm = cw == 24 ? 48 : knobs.chunk <= 16 ? 16 : knobs.chunk <= 24 ? 24 : 48;
+        if (!compiled(cw, maxm)) maxm = cw == 24 ? 48 : 24;
       }
       const int cpw = pipe_chunks_per_warp(cw), T = (n + maxm - 1) / maxm;
       if (!compiled(cw, maxm) || (T + cpw - 1) / cpw + extra > pipe_sm_warps(maxm)) continue;
