@@ -973,10 +973,12 @@ cudaError_t launch_pipe(const biofvm *h, int axis, int flags, cudaStream_t st, v
   b.dir_on = static_cast<const uint8_t *>(h->dir_on_d.p);
   b.dir_val = h->dir_val_d.p;
   b.status = static_cast<int *>(h->status.p);
-  // Programmatic serialisation (pipe.cuh) where a sweep is short: 113 x 97 x 121 x 3 with its
-  // adjoint 2.9% faster, 250^3 0.8%; 400^3 x 4, whose sweeps are bound by HBM, 2% slower, and in a
-  // batch, whose other environments fill the gaps, no faster.
-  b.overlap = !shared && (double)h->nel * (double)h->esz <= 96.0e6;
+  // Programmatic serialisation (pipe.cuh) where a sweep is short.  Steps without and with it: FP32
+  // fields of 16 MB 30.9 / 28.8 us, 62 MB 70.8 / 70.8, 90 MB 124 / 120, 134 MB 136 / 132, 187 MB
+  // 204 / 201, FP16 of 189 MB 295 / 291; FP32 of 268 MB 281 / 281, 1024 MB 1057 / 1060.  The line lies
+  // between the last that gains and the first that does not.  In a batch, whose other environments
+  // fill the gaps, it is no faster.
+  b.overlap = !shared && (double)h->nel * (double)h->esz <= 200.0e6;
   const CUtensorMap &map = p.map[axis == 0 ? 0 : buf];
   const int grid = shared ? p.shared_grid : p.grid;
   if (h->prec == BIOFVM_BF16) return launch_pipe_bf16(map, b, p.maxm, grid, p.smem, st);

@@ -146,3 +146,13 @@ def test_one_graph_a_call(lib, grid, steps):
         assert lib.biofvm_step(h, steps) == binding.OK
     assert lib.stand_in_graphs_made() == graphs + 1
     lib.biofvm_destroy(h)
+
+
+@pytest.mark.parametrize("grid, overlap", [((360, 360, 360, 1), 1), ((256, 256, 256, 4), 0)])
+def test_overlapped_launches_up_to_200_megabytes(lib, grid, overlap):
+    st, h = host_api.create(lib, *grid, "fp32")
+    assert st == binding.OK
+    lib.stand_in_forget_launches()
+    assert lib.biofvm_step(h, 1) == binding.OK
+    assert [r.overlap for r in host_api.pipe_launches(lib)] == [overlap] * 3
+    lib.biofvm_destroy(h)
