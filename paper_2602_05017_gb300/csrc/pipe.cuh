@@ -19,9 +19,8 @@
 //     instead of `full`;
 //   the next W warps (consumers): each thread holds one chunk (MAXM positions)
 //     of a PAIR of columns in registers and works on both with packed FP32
-//     instructions; a warp holds two chunks (CW = 16: four) of the
-//     tile's CW/2 pairs.
-//     Carries cross a warp by shuffles and the CTA through shared memory,
+//     instructions; a warp holds two chunks (CW = 16: four) of the tile's CW/2
+//     pairs (CW = 24: four lanes of each chunk's sixteen idle).  Carries cross a warp by shuffles and the CTA through shared memory,
 //     between two named barriers per tile that only consumers join.
 //
 // What bounds it.  One column per thread, coefficients and carry weights read
@@ -31,10 +30,11 @@
 // chunks whose coefficients have reached their interior values (all but the
 // first one or two and the last of a line) read none, and running the
 // recurrences again from the true carry replaces the correction passes: 16
-// instructions per element, all warps of the CTA counted.  Chunks are short (16 positions) because the
-// four dependent chains per tile are the remaining latency.  Measured, x / y /
-// z of 400^3 x 4: 0.540 / 0.506 / 0.513 ms before, 0.34 / 0.33 / 0.39 after
-// (HBM copy rate: 0.306); the z sweep's rows are 128 bytes, a plane apart.
+// instructions per element, all warps of the CTA counted.  Chunks are short (16
+// positions) because the four dependent chains per tile are the remaining
+// latency.  Measured, x / y / z of 400^3 x 4 with 1M agents: 0.540 / 0.506 / 0.513
+// ms before, 0.37 / 0.32 / 0.39 after (HBM copy rate: 0.306); the z sweep's rows
+// are 128 bytes, a plane apart.
 //
 // The grid is persistent (tiles strided by gridDim.x), so loads of later
 // tiles overlap the solve and the store of earlier ones.  The constants are
@@ -277,7 +277,10 @@ struct PairCoef : PairCoefBase {
   __device__ __forceinline__ ulonglong2 inv(int i) const { return Ti[i / 2]; }
   __device__ __forceinline__ ulonglong2 mul(int i) const { return Tm[i / 2]; }
 };
-// Each substrate's coefficients on their own (odd S, where the pairs would not fit).
+// Each substrate's coefficients on their own (odd S, where the pairs would not fit).  Four 8-byte
+// loads and the pairing moves in place of two 16-byte loads, in ragged chunks only: 64 x 1256 x 64 x 3
+// 94 us a step (the longest y line with pairs, 1240: 93), where other kernels took 283; 1072 x 64 x
+// 64 x 5 119 (285).
 template <>
 struct PairCoef<true> : PairCoefBase {
   const float *Ti0, *Ti1, *Tm0, *Tm1;  // of the pair's two substrates

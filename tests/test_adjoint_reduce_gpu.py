@@ -2,8 +2,9 @@
 same sums in numpy at 64 bits: lines around one and several segments of 32 positions, one voxel,
 substrate counts that do and do not divide a block, zeros, subnormals and infinities.
 
-Bound: FP64 products and sums, or (floats, eight at a time) pairs of floats of 48 bits: the result lies
-within (terms per sum) x 2^-53, or 8 x 2^-48, of the sum of the terms' sizes; 1e-13 covers both.
+Bound: FP64 sums, or floats eight at a time to no fewer bits: the result lies within (terms per sum)
+x 2^-53 of the sum of the terms' sizes, which 1e-13 covers (test_adjoint_reduce_bits_gpu.py holds
+them closer).
 """
 import ctypes
 

@@ -20,7 +20,7 @@ SHAPES = [
     (20, 21, 40, 5), (12, 40, 17, 9), (4, 33, 20, 32),      # odd counts, one row per tile
     (11, 4, 37, 1), (7, 8, 70, 3),                          # z tiles whose pairs cross rows
     (700, 3, 8, 4), (8, 704, 2, 1), (4, 2, 1300, 1),        # chunks of 24, 16-line tiles
-    (4, 730, 3, 1), (12, 4, 900, 2), (9, 8, 1000, 3),       # chunks of 48, 24-line tiles
+    (4, 730, 3, 1), (12, 4, 900, 2), (9, 8, 1000, 3),       # chunks of 48, 24 and 16 lines
 ]
 
 
