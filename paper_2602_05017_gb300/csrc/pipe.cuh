@@ -270,10 +270,6 @@ struct PairCoefBase {
 template <bool SPLIT>
 struct PairCoef : PairCoefBase {
   const ulonglong2 *Ti, *Tm;
-  __device__ __forceinline__ void at(const f2 *tab, int ncls, int npad, int cls, int, int, int lo) {
-    Ti = reinterpret_cast<const ulonglong2 *>(tab + cls * npad + lo);
-    Tm = reinterpret_cast<const ulonglong2 *>(tab + (ncls + cls) * npad + lo);
-  }
   __device__ __forceinline__ ulonglong2 inv(int i) const { return Ti[i / 2]; }
   __device__ __forceinline__ ulonglong2 mul(int i) const { return Tm[i / 2]; }
 };
@@ -284,12 +280,12 @@ struct PairCoef : PairCoefBase {
 template <>
 struct PairCoef<true> : PairCoefBase {
   const float *Ti0, *Ti1, *Tm0, *Tm1;  // of the pair's two substrates
-  __device__ __forceinline__ void at(const f2 *tab, int ncls, int npad, int, int sa, int sb, int lo) {
+  __device__ __forceinline__ void at(const f2 *tab, int S, int npad, int sa, int sb, int lo) {
     const float *const t = reinterpret_cast<const float *>(tab);
     Ti0 = t + sa * npad + lo;
     Ti1 = t + sb * npad + lo;
-    Tm0 = Ti0 + ncls * npad;  // (ncls == S)
-    Tm1 = Ti1 + ncls * npad;
+    Tm0 = Ti0 + S * npad;
+    Tm1 = Ti1 + S * npad;
   }
   static __device__ __forceinline__ ulonglong2 two(const float *a, const float *b) {
     const float2 x = *reinterpret_cast<const float2 *>(a), y = *reinterpret_cast<const float2 *>(b);
@@ -771,8 +767,15 @@ __global__ void __maxnreg__(pipe_regs(MAXM))
   auto set_substrates = [&](int sa, int sb) {
     const int cls = S == 1 ? 0 : S % 2 == 0 ? sa / 2 : sa;
     cf.K = tab + cls * 4;
-    cf.at(tab + 4 * ncls, ncls, npad, cls, sa, sb, lo);
-    const f2 *w = tab + 4 * ncls + (SPLIT ? 1 : 2) * ncls * npad;
+    const f2 *w;
+    if constexpr (SPLIT) {
+      cf.at(tab + 4 * ncls, S, npad, sa, sb, lo);
+      w = tab + 4 * ncls + ncls * npad;
+    } else {  // (each pointer from tab itself: from a common one 400^3 x 4 took 1059 us a step, so 1050)
+      cf.Ti = reinterpret_cast<const ulonglong2 *>(tab + 4 * ncls + cls * npad + lo);
+      cf.Tm = reinterpret_cast<const ulonglong2 *>(tab + 4 * ncls + (ncls + cls) * npad + lo);
+      w = tab + 4 * ncls + 2 * ncls * npad;
+    }
     cf.wt = w + (cls * (W * CPW) + t) * kWtN;
     cf.pw = w + ncls * (W * CPW) * kWtN + cls * W;
     dir.on0 = dir_after && a.dir_on[sa];
