@@ -178,7 +178,8 @@ struct biofvm {
   int reduce_blocks = 0;
   bool agents_on_device = false;
   std::vector<int64_t> h_voxel;
-  std::vector<int64_t> h_entry;  // per (agent, substrate): its element's source entry, or -1
+  std::vector<int64_t> h_entry;  // per (agent, substrate): its element's source entry, or -1; empty
+                                 // when the lists are (an upload failed)
   std::vector<double> h_weight, h_target;
   // the agents as last given (the source list is rebuilt when the nodes change)
   std::vector<double> h_secretion, h_uptake;
@@ -773,7 +774,8 @@ biofvm_status upload_constants(biofvm *h) {
               put(p0 + ((size_t)ncls + c) * npad + i, mul[(size_t)i * S + s]);
             }
           }
-          const size_t p1 = p0 + (size_t)(q.split ? S : 2 * ncls) * npad, p2 = p1 + (size_t)ncls * nch * kWtN;
+          const size_t p1 = p0 + (size_t)(q.split ? 1 : 2) * ncls * npad;
+          const size_t p2 = p1 + (size_t)ncls * nch * kWtN;
           for (int j = 0; j < nch; j++) {
             const int w = j / cpw;
             // product over chunks lo..hi within warp w
@@ -1288,7 +1290,7 @@ biofvm_status build_sources(biofvm *h) {
   CK(cudaStreamSynchronize(h->stream));  // the kernels may still read the old lists
   // Until every new list is on the device there is none, and no graph over buffers that go.
   h->n_entries = 0;
-  h->h_entry.assign((size_t)n * S, -1);
+  h->h_entry.clear();
   h->agents_on_device = false;  // the adjoint's agent-to-entry map follows the list
   h->generation++;
   drop_graphs(h);
@@ -2110,6 +2112,7 @@ biofvm_status biofvm_adjoint_step_rates(biofvm_t *h, const void *grad_out, void 
   const int64_t na = (int64_t)h->h_voxel.size();
   if (!h->agents_on_device && na > 0) {
     std::vector<int64_t> el((size_t)na * S);
+    if (h->h_entry.empty()) h->h_entry.assign((size_t)na * S, -1);
     const std::vector<int64_t> &en = h->h_entry;
     for (int64_t k = 0; k < na; k++)
       for (int s = 0; s < S; s++) el[k * S + s] = h->h_voxel[k] * S + s;
@@ -2338,10 +2341,11 @@ biofvm_status batch_capture_graph_mode(biofvm_batch *b, int K) {
 }
 
 // Per-environment mode: the environments' sweeps run side by side, so a sweep of the batch's own
-// step need not spread over every SM it can fill (a step of one environment's handle does).  With many tiles in all, at least four tiles a CTA: its constants
-// and the first tile's latency are then paid a quarter as often (20 environments of 64..128
-// voxels: 429 us a step with a CTA per tile where they fit, 365 with two tiles, 317 with four,
-// 335 with eight; two environments, 1014 tiles: 33.2, 32.3, 37.1 and 55.4).
+// step need not spread over every SM it can fill (a step of one environment's handle does).  With
+// many tiles in all, at least four tiles a CTA: its constants and the first tile's latency are then
+// paid a quarter as often (20 environments of 64..128 voxels: 429 us a step with a CTA per tile
+// where they fit, 365 with two tiles, 317 with four, 335 with eight; two environments, 1014 tiles:
+// 33.2, 32.3, 37.1 and 55.4).
 void batch_share_sms(biofvm_batch *b) {
   for (int axis = 0; axis < 3; axis++) {
     int64_t total = 0;
