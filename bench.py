@@ -45,18 +45,18 @@ HBM_FALLBACK_GBS = 6800.0
 # forward axpy + division, backward negated axpy).
 FLOPS_PER_ELEMENT_SWEEP = 5
 # Sources whose kernels the traffic below was captured on (hash of their contents).
-KERNEL_SOURCES = ["stream.cuh", "sweeps.cuh", "pipe.cuh", "pipe_args.h", "internal.h",
-                  "sweeps_fp64.cu", "sweeps_fp32.cu", "pipe_fp32.cu", "pipe_h16.cu", "api.cpp"]
+KERNEL_SOURCES = ["stream.cuh", "sweeps.cuh", "pipe.cuh", "pipe_args.h", "pipe_plan.h",
+                  "internal.h", "sweeps_fp64.cu", "sweeps_fp32.cu", "pipe_fp32.cu", "pipe_h16.cu", "api.cpp"]
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of each sweep kernel of
 # the 400^3 x 4 workload, from one ncu capture; reported only while the kernel sources still
 # hash to `sources_sha256` (otherwise the kernels changed since and traffic is null).
 MEASURED_TRAFFIC = {
-    "sources_sha256": "dfdfcfc5517b3db62d07efd51e965a28556916ae6b5369129c40901f2a165b99",
+    "sources_sha256": "b01f80e811e45226485df8271ba1a800e6cbbb503697a5e3bc9624dcc78edf1b",
     "bytes": {
-        "fp64:x-sweep": 5710992896, "fp64:y-sweep": 5504968192, "fp64:z-sweep": 5532824320,
-        "fp32:x-sweep": 2051157248, "fp32:y-sweep": 1983586816, "fp32:z-sweep": 1984059904,
-        "bf16:x-sweep": 1027370496, "bf16:y-sweep": 965999616, "bf16:z-sweep": 966979072,
-        "fp16:x-sweep": 1027427840, "fp16:y-sweep": 966120448, "fp16:z-sweep": 967207424,
+        "fp64:x-sweep": 5711458816, "fp64:y-sweep": 5528273664, "fp64:z-sweep": 5523283968,
+        "fp32:x-sweep": 2056011776, "fp32:y-sweep": 1991869184, "fp32:z-sweep": 1988227584,
+        "bf16:x-sweep": 1029618432, "bf16:y-sweep": 970411008, "bf16:z-sweep": 970359552,
+        "fp16:x-sweep": 1030117376, "fp16:y-sweep": 969882880, "fp16:z-sweep": 970134784,
     },
 }
 UNIT = "voxel-substrate updates/s"

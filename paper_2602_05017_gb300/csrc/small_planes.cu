@@ -1,6 +1,6 @@
 // Small grids with long lines (FP64): every step of a biofvm_step call in ONE
 // cooperative, persistent launch, the counterpart of small.cu for grids with a
-// line of more than 128 voxels (30 x 40 x 300 x 4: 71 us a step here, 101 there, where
+// line of more than 128 voxels (30 x 40 x 300 x 4: 68 us a step here, 101 there, where
 // such a line leaves an item one or two adjacent lines and each access a part of
 // a sector).
 //
